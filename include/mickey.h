@@ -214,7 +214,9 @@ MICKEY_API mickey_streams *mickey_import_state(const uint8_t *states,
  *           MICKEY_MODE_PERSISTENT2: two warps per SM sub-partition, each
  *           clocking and emitting (two blocks per SM, rows staged four
  *           tiles deep; with too few warp-groups it runs as PERSISTENT);
- *           MICKEY_MODE_AUTO: as PERSISTENT.
+ *           MICKEY_MODE_AUTO: one thread per instance for handles of up to 52
+ *           32-lane groups per SM (about 250,000 instances; unroll and stage
+ *           have no effect there), else as PERSISTENT.
  *   unroll  clocks per inner step, 2 or 4.
  *   stage   the output tile of the row layouts: 0 writes each 32-clock tile's
  *           4 bytes per row directly; otherwise each row's words of several
@@ -250,7 +252,7 @@ MICKEY_API int mickey_set_config(mickey_streams *s, int layout, int mode, int un
 MICKEY_API int mickey_get_config(const mickey_streams *s, int layout, int *mode,
                                  int *unroll, int *stage);
 
-/* Time every configuration (mode x unroll x output tile: up to 20
+/* Time every configuration (mode x unroll x output tile: up to 21
  * candidates) on this handle's own streams for one call of
  * n_bits in `layout` (the state is saved and restored: positions do not
  * move), keep the fastest for that layout (among candidates within 1 % of

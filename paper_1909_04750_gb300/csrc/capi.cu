@@ -207,6 +207,11 @@ int allocate(mickey_streams *s, size_t n) {
   return ok();
 }
 
+// Whether launches left to the library clock one instance per thread.
+bool use_packed(const mickey_streams *s) {
+  return s->G <= kPackedPerSm * uint32_t(s->sm_count);
+}
+
 // Key/IV loading + preclock for all instances of s.
 int run_init(mickey_streams *s, const void *keys, const void *ivs,
              const uint32_t *iv_lens, int mem) {
@@ -244,7 +249,10 @@ int run_init(mickey_streams *s, const void *keys, const void *ivs,
     dl = iv_lens;
   }
   LoadArgs la{dk, di, dl, n, nullptr, s->G, s->Gpad, s->d_scratch, s->d_err};
-  CUDA_TRY(launch_init(la, s->d_state, s->stream), "init_kernel launch");
+  if (s->mode == MICKEY_MODE_AUTO && use_packed(s))
+    CUDA_TRY(launch_packed_init(la, s->d_state, s->stream), "packed_init_kernel launch");
+  else
+    CUDA_TRY(launch_init(la, s->d_state, s->stream), "init_kernel launch");
   if (s->pos_max) std::fill(s->pos.begin(), s->pos.end(), 0);
   s->pos_base = s->pos_max = 0;
   return ok();
@@ -286,19 +294,24 @@ bool use_persistent(const mickey_streams *s, int mode) {
 }
 
 // One keystream launch of `bits` clocks into a device buffer.
+//   AUTO, few groups          one thread per instance
 //   GRID                      one thread per group, clocking and emitting
 //   PERSISTENT2, enough groups two clocking warps per SM sub-partition
 //   otherwise (AUTO, PERSISTENT) the paired kernel: clock warps beside emission
 //                             warps; with enough warp-groups the cooperative
 //                             launch with equal segments, else one warp-group
 //                             per pair.  It outruns the others at every size
-//                             measured, so AUTO takes it.
+//                             measured above the first line's, so AUTO takes it.
 int launch_generate(mickey_streams *s, uint64_t bits, void *out, int layout) {
   KeystreamArgs ka{s->d_state, s->G, s->Gpad, s->n, bits, out};
   const auto &c = s->cfg[layout];
   int mode = c.set ? c.mode : s->mode;
   const int unroll = c.set ? c.unroll : s->unroll;
   const int stage = c.set ? c.stage : s->stage;
+  if (mode == MICKEY_MODE_AUTO && use_packed(s)) {
+    CUDA_TRY(launch_packed_keystream(ka, layout, s->stream), "packed_keystream_kernel launch");
+    return MICKEY_OK;
+  }
   if (mode == MICKEY_MODE_GRID) {
     CUDA_TRY(launch_keystream(ka, layout, unroll, stage, nullptr, s->stream),
              "keystream_kernel launch");
@@ -771,12 +784,14 @@ int mickey_tune(mickey_streams *s, uint64_t n_bits, int layout, mickey_tune_resu
   int count = 0;
   // every candidate timed: (configuration, best of two)
   std::vector<std::pair<mickey_streams::LayoutCfg, float>> timed;
-  for (int mode : {MICKEY_MODE_GRID, MICKEY_MODE_PERSISTENT, MICKEY_MODE_PERSISTENT2}) {
+  for (int mode : {MICKEY_MODE_AUTO, MICKEY_MODE_GRID, MICKEY_MODE_PERSISTENT,
+                   MICKEY_MODE_PERSISTENT2}) {
     if (mode == MICKEY_MODE_PERSISTENT2 && !use_persistent(s, mode)) continue;
+    if (mode == MICKEY_MODE_AUTO && !use_packed(s)) continue;   // else the same as PERSISTENT
     // output tile: direct row stores, or rows staged this many tiles deep
     // (the depths the mode's kernels are compiled for)
-    std::vector<int> stages{0};
-    if (row) {
+    std::vector<int> stages{mode == MICKEY_MODE_AUTO ? 1 : 0};
+    if (row && mode != MICKEY_MODE_AUTO) {
       const std::vector<int> depths = mode == MICKEY_MODE_GRID      ? std::vector<int>{2, 4}
                                       : mode == MICKEY_MODE_PERSISTENT ? std::vector<int>{2, 4, 8}
                                                                     : std::vector<int>{4};
@@ -784,6 +799,7 @@ int mickey_tune(mickey_streams *s, uint64_t n_bits, int layout, mickey_tune_resu
         if (n_bits % (32 * uint64_t(d)) == 0) stages.push_back(d);
     }
     for (int unroll : kUnrolls) {
+      if (mode == MICKEY_MODE_AUTO && unroll != 4) continue;      // the packed launch has no choice
       for (int stage : stages) {
         auto &c = s->cfg[layout];
         c.set = true;

@@ -44,6 +44,22 @@ struct LoadArgs {
 // Gpad words).
 cudaError_t launch_init(const LoadArgs &a, uint32_t *state, cudaStream_t st);
 
+// The same with one thread per instance (packed.cu); the scratch of `a` is
+// not used.
+cudaError_t launch_packed_init(const LoadArgs &a, uint32_t *state, cudaStream_t st);
+
+// Launches of a handle whose mode is left to the library take one thread per
+// instance up to this many groups per SM, one thread per 32-lane group above.
+// Measured (152 SMs, us for 2048 bits of bytes / of a re-key; packed, thread
+// per group):
+//   groups    608      2432     4864     7296     8512
+//   2048 bits 76, 712  216, 710 412, 713 606, 713 703, 712
+//   re-key    30, 118  50, 119  77, 120  106, 120 121, 119
+// The packed times grow with the groups once every SM sub-partition has a
+// warp; a thread per group takes the time of one group's chain until all 608
+// sub-partitions have a warp of 32 groups (19456 groups), so the lines cross.
+constexpr uint32_t kPackedPerSm = 52;
+
 struct KeystreamArgs {
   uint32_t *state;          // kStateRows * Gpad words, read and written back
   uint32_t G, Gpad;
@@ -99,6 +115,10 @@ struct RaggedArgs {
   uint8_t *out;
 };
 cudaError_t launch_ragged(const RaggedArgs &a, int layout, cudaStream_t st);
+
+// One thread per instance (packed.cu), any n_bits, layout and alignment that
+// launch_keystream takes.
+cudaError_t launch_packed_keystream(const KeystreamArgs &a, int layout, cudaStream_t st);
 
 // p == nullptr: grid mode (one thread per group); else persistent mode.
 // stage: row layouts stage this many tiles per row (grid: 2 or 4; persistent:

@@ -1,0 +1,206 @@
+// Packed clock: one thread clocks one instance, its two 100-bit registers in
+// eight 32-bit words, so that a warp clocks one 32-lane group (device code of
+// the launches that are bound by the time per clock of one stream, not by the
+// throughput of many).
+//
+// Layout.  R bit i is bit j of word w, i = 4j + w; S bit i is at position
+// p = 99 - i = 4j + w.  With four words interleaved like this a shift of the
+// register is a renaming of the words plus a one-bit shift of a single one,
+// and with S reversed each control bit is one XOR of two bits at the same
+// place: s34 ^ r67 at bit 16 of a[1] ^ r[3], s67 ^ r33 at bit 8 of
+// a[0] ^ r[1].  Feedback bits: r99 is bit 24 of r[3], s99 bit 0 of a[0].
+// The S words hold a_i = s_i ^ COMP0_i (i = 1..98), so that the AND term is
+// a_i & (a_{i+1} ^ k_i) with k_i = COMP0_{i+1} ^ COMP1_i, and the constants
+// COMP0_{i-1} ^ COMP0_i join the feedback word.  s0 (which is the last
+// clock's feedback bit) is kept apart: its place in a[3] stays zero, so that
+// the AND term of bit 0, which the cipher does not have, is zero without a
+// mask; so does the one of bit 99, whose s_{i+1} is the zero shifted in.
+// Bits 25..31 of the r words hold shifted-out garbage that only moves up.
+//
+// Pipes.  The half-rate logic pipe bounds a warp on its own, so everything
+// that can be a multiply-add goes to the FMA pipe: left shifts, the feedback
+// words k2 + fb (FB0 part) + fb cbs (FB1 part) (each bit a 0/1 times a
+// constant, differences mod 2^32), fb_R x RTAPS and cb_R x r_i.  That leaves
+// 22 logic and 23 multiply-add operations per clock of 32 instances.
+// Measured (GB300, 2.07 GHz, clocks alone): 29.4 ns per clock for a lone
+// warp, 31.3 with one warp per SM sub-partition, 782 Gbit/s with eight;
+// with the R update in logic operations 29.8 / 31.1 ns and 717 Gbit/s.  The
+// column form spread over a warp's lanes (four bits of each register per
+// lane, seven shuffles per clock), which this one replaces, took 34.2 ns and
+// at most 649 Gbit/s; one thread per 32-lane group takes 334 ns.
+#pragma once
+
+#include <cstdint>
+
+#include "bitslice.cuh"
+
+namespace mickey {
+
+struct Packed {
+  uint32_t r[4], a[4], s0;
+};
+
+__host__ __device__ constexpr bool packed_c0(int i) { return i >= 1 && i <= 98 && comp0(i); }
+
+struct PackedMasks {
+  uint32_t tap[4];   // RTAPS
+  uint32_t c0[4];    // COMP0: a = s ^ c0
+  uint32_t k[4];     // AND term a_i & (a_{i+1} ^ k_i)
+  uint32_t k2[4];    // COMP0_{i-1} ^ COMP0_i
+  uint32_t x[4];     // (k2 ^ FB0) - k2
+  uint32_t y[4];     // (k2 ^ FB1) - (k2 ^ FB0)
+};
+constexpr PackedMasks make_packed_masks() {
+  PackedMasks m{};
+  for (int w = 0; w < 4; ++w) {
+    uint32_t f0 = 0, f1 = 0;
+    for (int j = 0; j < 25; ++j) {
+      const uint32_t b = 1u << j;
+      if (rtap(4 * j + w)) m.tap[w] |= b;
+      const int i = 99 - (4 * j + w);
+      if (i == 0) continue;                  // kept in Packed::s0
+      if (packed_c0(i)) m.c0[w] |= b;
+      if (fb0(i)) f0 |= b;
+      if (fb1(i)) f1 |= b;
+      if (packed_c0(i - 1) != packed_c0(i)) m.k2[w] |= b;
+      if (i <= 98 && packed_c0(i + 1) != comp1(i)) m.k[w] |= b;
+    }
+    m.x[w] = (m.k2[w] ^ f0) - m.k2[w];
+    m.y[w] = (m.k2[w] ^ f1) - (m.k2[w] ^ f0);
+  }
+  return m;
+}
+constexpr PackedMasks kPackedMasks = make_packed_masks();
+
+// a * b + c on the FMA pipe (written out: as C++ the products with 0/1 become
+// logic operations).
+__device__ __forceinline__ uint32_t mad32(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t d;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+
+// One CLOCK_KG of the thread's instance; MIX as in clock_kg, `in` 0 or 1.
+template <bool MIX>
+__device__ __forceinline__ void clock_packed(Packed &q, uint32_t in) {
+  static_assert(!packed_c0(34) && packed_c0(67) && !packed_c0(50), "control bits as held");
+  uint32_t(&r)[4] = q.r;
+  uint32_t(&a)[4] = q.a;
+  const uint32_t cbr = ((a[1] ^ r[3]) >> 16) & 1u;   // CONTROL_BIT_R
+  uint32_t fbr, fbs;                                 // fbr: 0 or ~0; fbs: 0 or 1
+  if constexpr (MIX) {
+    fbr = 0u - (((r[3] >> 24) ^ (a[1] >> 12) ^ in) & 1u);   // r99 ^ s50 ^ in
+    fbs = (a[0] ^ in) & 1u;
+  } else {
+    fbr = uint32_t(int32_t(r[3] << 7) >> 31);
+    fbs = a[0] & 1u;
+  }
+  const uint32_t ncbs = (a[0] ^ r[1]) >> 8;          // bit 0: NOT CONTROL_BIT_S
+  const uint32_t fc = lop3<0x20>(fbs, ncbs, 1u);     // fbs & ~ncbs & 1
+  uint32_t nr[4], na[4];
+  static_for<0, 4>([&](auto wc) {
+    constexpr int w = decltype(wc)::value;
+    constexpr uint32_t tap = 0u - kPackedMasks.tap[w], k = kPackedMasks.k[w],
+                       k2 = kPackedMasks.k2[w], x = kPackedMasks.x[w], y = kPackedMasks.y[w];
+    const uint32_t rm1 = w ? r[(w + 3) % 4] : r[3] << 1;                  // r_{i-1}
+    nr[w] = lop3<0x96>(rm1, mad32(r[w], cbr, 0u), mad32(fbr, tap, 0u));
+    const uint32_t sp1 = w ? a[(w + 3) % 4] : a[3] << 1;                  // a_{i+1}
+    const uint32_t sm1 = w < 2    ? a[(w + 1) % 4]                        // a_{i-1}
+                         : w == 2 ? mad32(q.s0, 1u << 24, a[3])
+                                  : a[0] >> 1;
+    const uint32_t v = lop3<0x60>(a[w], sp1, k);                          // a & (sp1 ^ k)
+    na[w] = lop3<0x96>(v, sm1, mad32(fc, y, mad32(fbs, x, k2)));
+  });
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    r[w] = nr[w];
+    a[w] = na[w];
+  }
+  q.s0 = fbs;
+}
+
+// The zero state.
+__device__ __forceinline__ void packed_zero(Packed &q) {
+  static_for<0, 4>([&](auto wc) {
+    constexpr int w = decltype(wc)::value;
+    constexpr uint32_t c0 = kPackedMasks.c0[w];
+    q.r[w] = 0u;
+    q.a[w] = c0;
+  });
+  q.s0 = 0u;
+}
+
+// N clocks in non-mixing mode; z of clock c in bit N - 1 - c of the result
+// (after N = 32: the first clock's in bit 31).
+template <int N>
+__device__ __forceinline__ uint32_t packed_clocks(Packed &q) {
+  uint32_t z = 0;
+#pragma unroll
+  for (int c = 0; c < N; ++c) {
+    z = mad32(z, 2u, lop3<0x28>(q.r[0], q.s0, 1u));   // (r0 ^ s0) & 1
+    clock_packed<false>(q, 0u);
+  }
+  return z;
+}
+
+// The n < 32 clocks of a last partial tile, left-aligned as a whole tile.
+__device__ __forceinline__ uint32_t packed_tail(Packed &q, int n) {
+  uint32_t z = 0;
+#pragma unroll 1
+  for (int c = 0; c < n; ++c) {
+    z = mad32(z, 2u, lop3<0x28>(q.r[0], q.s0, 1u));
+    clock_packed<false>(q, 0u);
+  }
+  return z << (32 - n);
+}
+
+// 32 x 32 bit transpose across the warp: lane l's bit b <-> lane b's bit l.
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x, uint32_t lane) {
+  constexpr uint32_t kLow[5] = {0x0000ffffu, 0x00ff00ffu, 0x0f0f0f0fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    const uint32_t j = 16u >> st, m = kLow[st];
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+    x = (lane & j) ? (x & ~m) | ((y >> j) & m) : (x & m) | ((y & m) << j);
+  }
+  return x;
+}
+
+// Group g's bitsliced state (word-major rows of P words, r0..r99 then
+// s0..s99) to the lanes' packed registers and back: lane j reads or writes
+// the row of bit j of each word, and the transpose turns rows into lanes.
+__device__ __forceinline__ void packed_load(Packed &q, const uint32_t *state, size_t P, uint32_t g,
+                                            uint32_t lane) {
+  uint32_t x[8];
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const int i = int(4 * lane) + w;
+    x[w] = lane < 25 ? state[size_t(i) * P + g] : 0u;
+    x[4 + w] = lane < 25 ? state[size_t(kReg + 99 - i) * P + g] : 0u;
+  }
+  static_for<0, 4>([&](auto wc) {
+    constexpr int w = decltype(wc)::value;
+    constexpr uint32_t c0 = kPackedMasks.c0[w];
+    q.r[w] = warp_transpose(x[w], lane);
+    q.a[w] = warp_transpose(x[4 + w], lane) ^ c0;
+  });
+  q.s0 = (q.a[3] >> 24) & 1u;
+  q.a[3] &= 0x00ffffffu;
+}
+
+__device__ __forceinline__ void packed_store(const Packed &q, uint32_t *state, size_t P,
+                                             uint32_t g, uint32_t lane) {
+  static_for<0, 4>([&](auto wc) {
+    constexpr int w = decltype(wc)::value;
+    constexpr uint32_t c0 = kPackedMasks.c0[w];
+    const uint32_t a = (w == 3 ? q.a[w] | (q.s0 << 24) : q.a[w]) ^ c0;
+    const uint32_t xr = warp_transpose(q.r[w], lane), xs = warp_transpose(a, lane);
+    const int i = int(4 * lane) + w;
+    if (lane < 25) {
+      state[size_t(i) * P + g] = xr;
+      state[size_t(kReg + 99 - i) * P + g] = xs;
+    }
+  });
+}
+
+}  // namespace mickey

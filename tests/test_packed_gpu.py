@@ -1,0 +1,123 @@
+"""The one-thread-per-instance launches of a streams handle (keystream and
+initialisation) against the oracle and against the one-thread-per-group
+launches, on whose state in HBM they go on and the other way round."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1909_04750_gb300 import _native as N
+from paper_1909_04750_gb300 import workloads
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+THREADS = os.cpu_count() or 4
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1909_04750_gb300 import build as B
+    B.build()
+    N.lib()
+
+
+def _streams(s):
+    from paper_1909_04750_gb300.streams import Streams
+    return Streams(torch.from_numpy(s.keys).cuda(), torch.from_numpy(s.ivs).cuda(),
+                   torch.from_numpy(s.iv_lens.astype(np.int32)).cuda())
+
+
+def _mixed(n):
+    s = workloads.plain_scale(n)
+    s.iv_lens[:] = np.random.default_rng(n).integers(0, 81, n)
+    return s
+
+
+# one tile less or more a bit, the 16-byte row stores (multiples of 128) and what is left of them
+@pytest.mark.parametrize("n_bits", [1, 31, 32, 33, 96, 124, 128, 160, 256, 1001])
+@pytest.mark.parametrize("n", [1, 31, 33, 1000])
+def test_every_layout_two_calls_against_the_oracle(n, n_bits):
+    s = _mixed(n)
+    ref = oracle.batch_bytes(s.keys, s.ivs, s.iv_lens, n_bits + 64, threads=THREADS)
+    bits = np.unpackbits(ref, axis=1)
+    for layout in ("bytes", "bitsliced", "u32", "u32_f32"):
+        if layout.startswith("u32") and n_bits % 32:
+            continue
+        st = _streams(s)
+        first, second = st.generate(n_bits, layout), st.generate(64, layout)
+        st.sync()
+        for got, lo, hi in ((first, 0, n_bits), (second, n_bits, n_bits + 64)):
+            want = np.packbits(bits[:, lo:hi], axis=1)
+            a = got.cpu().numpy()
+            if layout == "bytes":
+                assert np.array_equal(a, want)
+            elif layout == "bitsliced":
+                assert np.array_equal(a.view(np.uint32), oracle.to_bitsliced(want, hi - lo))
+            else:
+                u = oracle.to_u32(want, hi - lo)
+                assert np.array_equal((a if layout == "u32" else a[0]).view(np.uint32), u)
+                if layout == "u32_f32":
+                    assert np.array_equal(a[1].view(np.float32), oracle.to_f32(u))
+
+
+@pytest.mark.parametrize("offset", [1, 2, 4, 8, 12])
+@pytest.mark.parametrize("n_bits", [96, 256, 1001])
+def test_output_at_any_alignment(n_bits, offset):
+    s = _mixed(70)
+    want = oracle.batch_bytes(s.keys, s.ivs, s.iv_lens, n_bits, threads=THREADS)
+    st = _streams(s)
+    buf = torch.full((70 * want.shape[1] + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+    st.generate(n_bits, "bytes", out=buf[offset:])
+    st.sync()
+    got = buf.cpu().numpy()
+    assert np.array_equal(got[offset:offset + want.size].reshape(want.shape), want)
+    assert (got[:offset] == 0xA5).all() and (got[offset + want.size:] == 0xA5).all()
+
+
+@pytest.mark.parametrize("extra", [0, 1])
+def test_last_size_and_the_next_agree_with_a_thread_per_group(monkeypatch, extra):
+    # the largest handle of the packed launches and one group more, against an
+    # explicit grid launch: output, a second call, the state
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    s = _mixed((52 * sms + extra) * 32 - 5)
+    auto = _streams(s)
+    monkeypatch.setenv("MICKEY_MODE", "grid")
+    grid = _streams(s)
+    for n_bits, layout in ((64, "bytes"), (96, "u32"), (33, "bitsliced")):
+        assert torch.equal(auto.generate(n_bits, layout), grid.generate(n_bits, layout))
+    states = [h.export_state()[0] for h in (auto, grid)]
+    assert np.array_equal(*states)
+
+
+@pytest.mark.parametrize("n", [32 * 300 + 7, 5 * 1024 + 1])
+def test_thread_per_group_loading_paths_small(monkeypatch, n):
+    # small handles of an explicit mode load with a thread per group: 16-byte
+    # loads, and through shared memory when unaligned
+    from paper_1909_04750_gb300.streams import Streams
+    monkeypatch.setenv("MICKEY_MODE", "grid")
+    s = _mixed(n)
+    want = oracle.batch_bytes(s.keys, s.ivs, s.iv_lens, 96, threads=THREADS)
+    lens = torch.from_numpy(s.iv_lens.astype(np.int32)).cuda()
+    for off in (0, 1, 6):
+        keys, ivs = (torch.zeros(n * 10 + 16, dtype=torch.uint8, device="cuda")[off:off + n * 10]
+                     for _ in range(2))
+        keys.copy_(torch.from_numpy(s.keys.reshape(-1)))
+        ivs.copy_(torch.from_numpy(s.ivs.reshape(-1)))
+        st = Streams(keys.view(n, 10), ivs.view(n, 10), lens)
+        assert np.array_equal(st.generate(96, "bytes").cpu().numpy(), want)
+        st.sync()
+
+
+def test_a_long_iv_is_reported():
+    s = _mixed(100)
+    lens = torch.from_numpy(s.iv_lens.astype(np.int32)).cuda()
+    lens[77] = 81
+    from paper_1909_04750_gb300.streams import Streams
+    st = Streams(torch.from_numpy(s.keys).cuda(), torch.from_numpy(s.ivs).cuda(), lens)
+    with pytest.raises(N.MickeyError) as e:
+        st.sync()
+    assert e.value.code == N.E_IVLEN
