@@ -299,9 +299,10 @@ MICKEY_API int mickey_batch_run(mickey_batch *b, const void *keys, const void *i
 /* Launch configuration of the batch's keystream kernel: clocks per inner
  * step (2 or 4), resident blocks of 4 warps per SM (1 or 2), and
  * split_clocks: groups needing more clocks than this are each run by a whole
- * warp (lane j clocks register bits 4j..4j+3, about ten times less time per
- * clock, for long streams whose sequential clocks bound the run); 0 disables
- * the split path.  Re-captures the graph. */
+ * warp, a stream per lane (about ten times less time per clock than a thread
+ * per group, for long streams whose sequential clocks bound the run); 0
+ * disables the split path.  A new plan of up to 400 groups per SM splits
+ * every group (split_clocks 1), a larger one none.  Re-captures the graph. */
 MICKEY_API int mickey_batch_set_config(mickey_batch *b, int unroll, int blocks_per_sm,
                                        uint64_t split_clocks);
 /* Where the split groups run (re-captures the graph):

@@ -129,6 +129,7 @@ def tune(batch: Batch, keys, ivs, out: torch.Tensor, refresh: bool = False) -> d
         for sc in ((0,) if mx <= 1 << 16 else ()) + (mx // 4, mx // 8, mx // 16, mx // 32,
                                                      mx // 64):
             trial(4, b, sc)
+    trial(4, 1, 1)      # every group split, as a new plan of up to 400 groups per SM has it
     best = min(cands, key=lambda c: c["ms"])
     trial(2, best["blocks_per_sm"], best["split_clocks"])
     best = min(cands, key=lambda c: c["ms"])

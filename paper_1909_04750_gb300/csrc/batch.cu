@@ -10,9 +10,9 @@
 //
 // Run (device, captured once as a CUDA graph and replayed): key/IV loading
 // through the sorting permutation, preclock, then the keystream.  The first
-// n_split groups, the longest, run one per warp (split path: the warp clocks
-// one group, several times less time per clock, for the groups that bound
-// the run); the rest 32 consecutive groups per warp item, one per thread.
+// n_split groups, the longest, run one per warp (split path: a stream per
+// lane, many times less time per clock, for the groups that bound the run);
+// the rest 32 consecutive groups per warp item, one per thread.
 // Items are taken from atomic counters longest first (longest processing
 // time first).  Two arrangements (the split mode):
 //   shared  one persistent kernel: its warps take the split items first,
@@ -35,7 +35,7 @@
 #include "../../include/mickey.h"
 #include "bitslice.cuh"
 #include "internal.h"
-#include "split.cuh"
+#include "packed.cuh"
 
 using namespace mickey;
 
@@ -178,43 +178,41 @@ __device__ __forceinline__ void store_row(uint8_t *o, uint64_t bits, uint32_t t,
   for (int b = 0; b < nbytes; ++b) o[b] = uint8_t(w >> (8 * b));
 }
 
-// One warp per group (split path).  Not inlined: as a function of its own it
-// gets a register allocation of its own (about 120 registers, no spills)
-// instead of sharing the one-thread-per-group path's 255, which made its
-// clock about 20 % slower.  The tile's bits come back transposed
-// (clock c in bit c of lane l's word), reversed so that the tile's first
-// clock comes first, and put in memory byte order.
-__device__ __noinline__ void split_group(const uint32_t *state, size_t P, uint32_t g,
-                                            uint64_t clocks, uint8_t *row, uint64_t bits,
-                                            uint32_t lane, uint32_t *zbuf0, uint32_t *zbuf1) {
-  SplitLane k;
-  split_lane_init(lane, k);
-  uint32_t r[4], s[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int i = int(4 * lane) + q;
-    r[q] = i < kReg ? state[size_t(i) * P + g] : 0u;
-    const int is = split_s_bit(int(lane), q);
-    s[q] = is >= 0 && is < kReg ? state[size_t(kReg + is) * P + g] : 0u;
-  }
+// One warp per group (split path), a stream per lane (packed.cuh): the group
+// runs as long as its longest lane.  Rows that start 16-byte aligned are
+// written four tiles at a time while the lane has them whole.  Not inlined:
+// as a function of its own it gets a register allocation of its own instead
+// of sharing the one-thread-per-group path's 255.
+__device__ __noinline__ void packed_group(const uint32_t *state, size_t P, uint32_t g,
+                                          uint64_t clocks, uint8_t *row, uint64_t bits,
+                                          uint32_t lane) {
+  Packed q;
+  packed_load(q, state, P, g, lane);
   const uint32_t full = uint32_t(clocks >> 5);
+  const bool vec = (reinterpret_cast<uintptr_t>(row) & 15u) == 0;
+  uint4 v = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
   for (uint32_t t = 0; t < full; ++t) {
-    const uint32_t mine = split_tile<kSplitUnroll>(r, s, k, lane, zbuf0, zbuf1, 32);
-    store_row(row, bits, t, __byte_perm(__brev(mine), 0u, 0x0123));
+    const uint32_t w = __byte_perm(packed_clocks<32>(q), 0u, 0x0123);
+    v = make_uint4(v.y, v.z, v.w, w);
+    if (!vec) {
+      store_row(row, bits, t, w);
+    } else if ((t & 3) == 3 && (uint64_t(t) + 1) * 32 <= bits) {
+      *reinterpret_cast<uint4 *>(row + 4ull * (t - 3)) = v;
+    } else if ((t & 3) == 3 || t == full - 1) {   // a block of four that ends early
+      const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (uint32_t j = 0; j < 4; ++j)
+        if (3 - j <= (t & 3)) store_row(row, bits, t - (3 - j), w4[j]);
+    }
   }
   const int rem = int(clocks & 31);
-  if (rem) {
-    const uint32_t mine = split_tile<kSplitUnroll>(r, s, k, lane, zbuf0, zbuf1, rem);
-    store_row(row, bits, full, __byte_perm(__brev(mine), 0u, 0x0123));
-  }
-  __syncwarp();
+  if (rem) store_row(row, bits, full, __byte_perm(packed_tail(q, rem), 0u, 0x0123));
 }
 
 // Split kernel: one-warp blocks take the split groups (0 .. n_split-1,
 // longest first) one at a time.
 __global__ void __launch_bounds__(32) batch_split_kernel(BatchArgs a) {
-  __shared__ uint32_t zs[64];
   const uint32_t lane = threadIdx.x;
   uint8_t *out = a.params->out;
 #pragma unroll 1
@@ -224,8 +222,8 @@ __global__ void __launch_bounds__(32) batch_split_kernel(BatchArgs a) {
     item = __shfl_sync(0xffffffffu, item, 0);
     if (item >= a.n_split) break;
     const uint64_t slot = uint64_t(item) * 32 + lane;
-    split_group(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
-                a.slot_bits[slot], lane, zs, zs + 32);
+    packed_group(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
+                 a.slot_bits[slot], lane);
   }
 }
 
@@ -244,11 +242,9 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(BatchArgs a) {
     item = __shfl_sync(0xffffffffu, item, 0);
     if (item >= a.n_items) break;
     if (item < a.split_items) {
-      // the warp's own 32 columns of rows 0 and 1 of the tile buffer
       const uint64_t slot = uint64_t(item) * 32 + lane;
-      uint32_t *zb = zs + (threadIdx.x & ~31u);
-      split_group(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
-                  a.slot_bits[slot], lane, zb, zb + kBatchThreads);
+      packed_group(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
+                   a.slot_bits[slot], lane);
       continue;
     }
     const uint32_t g = a.n_split + (item - a.split_items) * 32 + lane;
@@ -273,6 +269,7 @@ struct mickey_batch {
   uint64_t split_clocks = 0;      // groups longer than this use the split path (0: none)
   uint32_t n_split = 0;
   int split_mode = MICKEY_BATCH_SPLIT_SHARED;
+  int split_warps = 1;            // warps per SM sub-partition when every group is split
   // device
   uint8_t *d_in = nullptr;        // keys (10n), ivs (10n), iv_lens (4n) in caller order
   uint32_t *d_perm = nullptr;     // 32*Gpad
@@ -302,6 +299,37 @@ void batch_release(mickey_batch *b) {
   delete b;
 }
 
+// Time per clock (ns) of a split warp when 1, 2, 3 or 4 share an SM
+// sub-partition (row stores included).
+constexpr double kPackedNs[4] = {32.0, 55.0, 78.0, 102.0};
+// Up to this many groups per SM a new plan splits every group.  A thread item
+// clocks 32 groups at 820 ns per clock (1140 when two share a sub-partition),
+// so it wins only once there are items for every warp and their lengths are
+// alike.  Measured, all split against the best of no split (ms): 20,000
+// streams of 2^10..2^18 bits 8.6, 158; 100,000 of 2^10..2^22 138, 2860;
+// 700,000 of 2^13 7.57, 9.99; 1.5 M of 2^12 8.32, 8.95; 4 M of 2^10..2^13
+// 18.5, 17.9.
+constexpr uint32_t kSplitAllPerSm = 400;
+
+// The arrangement of a new plan: all groups split, with as many warps per SM
+// sub-partition as finish first (few while the longest group's chain is what
+// takes the time, more when the groups have to share the chip anyway).
+void plan_split(mickey_batch *b) {
+  if (b->G <= kSplitAllPerSm * uint32_t(b->sm_count)) {
+    b->split_clocks = 1;
+    b->n_split = b->G;
+  }
+  double best = 1e300;
+  for (int k = 0; k < 4; ++k) {
+    const double t = std::max(double(b->max_clocks) * kPackedNs[k],
+                              double(b->total_clocks) * kPackedNs[k] / ((k + 1) * 4.0 * b->sm_count));
+    if (t < best) {
+      best = t;
+      b->split_warps = k + 1;
+    }
+  }
+}
+
 // Capture load + preclock, then the split kernel and the thread kernel as
 // two parallel branches, into a graph.
 cudaError_t capture(mickey_batch *b) {
@@ -321,8 +349,12 @@ cudaError_t capture(mickey_batch *b) {
     cudaMemsetAsync(b->d_queue, 0, 2 * sizeof(uint32_t), cs);
     LoadArgs la{b->d_in, b->d_in + 10 * n, reinterpret_cast<const uint32_t *>(b->d_in + 20 * n),
                 n, b->d_perm, b->G, b->Gpad, b->d_scratch, b->d_err};
-    launch_init(la, b->d_state, cs);
-    const bool own = b->split_mode == MICKEY_BATCH_SPLIT_OWN && b->n_split;
+    if (b->G <= kPackedPerSm * uint32_t(b->sm_count))
+      launch_packed_init(la, b->d_state, cs);
+    else
+      launch_init(la, b->d_state, cs);
+    // without thread items the split kernel is all there is, whatever the mode
+    const bool own = b->n_split && (b->split_mode == MICKEY_BATCH_SPLIT_OWN || b->n_split == b->G);
     const uint32_t split_items = own ? 0u : b->n_split;
     BatchArgs ba{b->d_state, b->G, b->Gpad, b->d_slot, b->d_slot + 32 * size_t(b->Gpad),
                  b->d_slot + 64 * size_t(b->Gpad), b->n_split, split_items,
@@ -330,7 +362,8 @@ cudaError_t capture(mickey_batch *b) {
     if (own) {   // the split groups on a branch of their own
       cudaEventRecord(fork, cs);
       cudaStreamWaitEvent(cs2, fork, 0);
-      const uint32_t warps = std::min<uint32_t>(b->n_split, uint32_t(b->sm_count) * 4u);
+      const uint32_t per = b->n_split == b->G ? uint32_t(b->split_warps) : 1u;
+      const uint32_t warps = std::min<uint32_t>(b->n_split, uint32_t(b->sm_count) * 4u * per);
       batch_split_kernel<<<warps, 32, 0, cs2>>>(ba);
       cudaEventRecord(join, cs2);
     }
@@ -422,6 +455,7 @@ MICKEY_API mickey_batch *mickey_batch_create(const uint32_t *iv_lens, const uint
     b->total_clocks += c;
     b->max_clocks = std::max(b->max_clocks, c);
   }
+  plan_split(b);
   bool ok = cudaMalloc(&b->d_in, 24 * n) == cudaSuccess &&
             cudaMalloc(&b->d_perm, slots * 4) == cudaSuccess &&
             cudaMalloc(&b->d_slot, slot.size() * 8) == cudaSuccess &&

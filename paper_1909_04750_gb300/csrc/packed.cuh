@@ -203,4 +203,40 @@ __device__ __forceinline__ void packed_store(const Packed &q, uint32_t *state, s
   });
 }
 
+// A row of register bits in order, bit i at bit 31 - i % 32 of word i / 32
+// (R in words 0..3, S in 4..7), to the packed registers and back.
+__device__ __forceinline__ void packed_from_row(Packed &q, const uint32_t (&row)[8]) {
+  static_for<0, 4>([&](auto wc) {
+    constexpr int w = decltype(wc)::value;
+    constexpr uint32_t c0 = kPackedMasks.c0[w];
+    uint32_t r = 0u, s = 0u;
+#pragma unroll
+    for (int j = 0; j < 25; ++j) {
+      const int i = 4 * j + w, k = 99 - i;
+      r |= ((row[i >> 5] >> (31 - (i & 31))) & 1u) << j;
+      s |= ((row[4 + (k >> 5)] >> (31 - (k & 31))) & 1u) << j;
+    }
+    q.r[w] = r;
+    q.a[w] = s ^ c0;
+  });
+  q.s0 = (q.a[3] >> 24) & 1u;
+  q.a[3] &= 0x00ffffffu;
+}
+
+__device__ __forceinline__ void packed_to_row(const Packed &q, uint32_t (&row)[8]) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) row[k] = 0u;
+  static_for<0, 4>([&](auto wc) {
+    constexpr int w = decltype(wc)::value;
+    constexpr uint32_t c0 = kPackedMasks.c0[w];
+    const uint32_t a = (w == 3 ? q.a[w] | (q.s0 << 24) : q.a[w]) ^ c0;
+#pragma unroll
+    for (int j = 0; j < 25; ++j) {
+      const int i = 4 * j + w, k = 99 - i;
+      row[i >> 5] |= ((q.r[w] >> j) & 1u) << (31 - (i & 31));
+      row[4 + (k >> 5)] |= ((a >> j) & 1u) << (31 - (k & 31));
+    }
+  });
+}
+
 }  // namespace mickey

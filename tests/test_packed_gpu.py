@@ -121,3 +121,26 @@ def test_a_long_iv_is_reported():
     with pytest.raises(N.MickeyError) as e:
         st.sync()
     assert e.value.code == N.E_IVLEN
+
+
+@pytest.mark.parametrize("offset", [0, 4])
+def test_new_batch_plan_row_ends_at_any_tile(offset):
+    # every group split; rows of one group end inside and at the ends of tiles
+    # and of the four-tile row stores, with 16- and 4-byte aligned rows
+    from paper_1909_04750_gb300.batch import Batch
+    s = _mixed(200)
+    nb = np.arange(200, dtype=np.uint64) * 3
+    nb[:10] = [0, 1, 31, 32, 33, 127, 128, 129, 256, 4096]
+    b = Batch(nb, s.iv_lens)
+    assert b.get_config()["split_groups"] == 7
+    buf = torch.full((b.output_bytes + 16,), 0xA5, dtype=torch.uint8, device="cuda")
+    out = b.run(torch.from_numpy(s.keys).cuda(), torch.from_numpy(s.ivs).cuda(), buf[offset:])
+    b.sync()
+    want = oracle.batch_bytes(s.keys, s.ivs, s.iv_lens, nb, threads=THREADS)
+    for got, row in zip(b.rows(out), want):
+        assert np.array_equal(got, np.asarray(row)[:got.size])
+    host = out.cpu().numpy()
+    used = np.zeros(host.size, bool)
+    for o, n in zip(b.offsets, nb):
+        used[int(o):int(o) + (int(n) + 7) // 8] = True
+    assert (host[~used] == 0xA5).all()
