@@ -24,8 +24,11 @@
  *           launch takes (warp-group, 1280-clock chunk) items from a queue,
  *           each chunk continuing from the state its predecessor published
  *           (a bounded wait: MICKEY_SPIN_LIMIT polls of about 256 ns, after
- *           which grain_sync reports MICKEY_E_TIMEOUT).  MICKEY_GRAIN_QUEUE=1,
- *           read when a handle is created, forces the queue.  The bytes
+ *           which grain_sync reports MICKEY_E_TIMEOUT).  Handles with few
+ *           groups (bitsliced up to 110 per SM, bytes up to 180 or any
+ *           number when rows are not 16-byte aligned) run one thread per
+ *           instance instead.  MICKEY_GRAIN_QUEUE, read when a handle is
+ *           created: 1 forces the queue, 0 the warp per warp-group.  The bytes
  *           layout stages rows in tensor memory (one block of 8 warps per SM).
  */
 #ifndef GRAIN_H

@@ -570,7 +570,8 @@ struct grain_streams {
   int sm_count = 0;
   uint32_t spin_limit = 1u << 24;
   int force = -1;                // MICKEY_GRAIN_QUEUE=1: always the queue-fed launch,
-                                 // =0 (the default): the grid launch when every warp-group fits
+                                 // =0: the grid launch when every warp-group fits;
+                                 // neither: one thread per instance for few groups, else as 0
 };
 
 namespace {
@@ -585,6 +586,31 @@ void grain_release(grain_streams *s) {
   cudaFree(s->d_queue);
   cudaFree(s->d_err);
   delete s;
+}
+
+// Up to how many groups per SM a launch left to the library takes one thread
+// per instance.  Measured (152 SMs; us; packed, thread per group):
+//   groups                       126      4864       14592      19456      32768
+//   bitsliced, 10002 bits     47, 743   281, 746   815, 969  1080, 978  1815, 1311
+//   bytes, 8192 bits          44, 889   204, 1025  572, 1113  757, 1146  1265, 1213
+//   initialisation            11, 28    15, 29     25, 30     31, 31     44, 35
+// The packed launches' work grows with the groups from one warp per SM
+// sub-partition on; a thread per group takes one warp-group's chain until
+// every sub-partition has two.
+constexpr uint32_t kGrainPackedInitPerSm = 128;
+constexpr uint32_t kGrainPackedBitslicedPerSm = 110, kGrainPackedBytesPerSm = 180;
+
+bool grain_use_packed(const grain_streams *s, uint32_t per_sm) {
+  return s->force < 0 && s->G <= per_sm * uint32_t(s->sm_count);
+}
+
+// Loading and initialisation clocks from device inputs.
+cudaError_t grain_init(const grain_streams *s, const uint8_t *dk, const uint8_t *dv) {
+  if (grain_use_packed(s, kGrainPackedInitPerSm))
+    return launch_grain_packed_init(dk, dv, s->n, s->G, s->Gpad, s->d_state, s->stream);
+  GrainInitArgs ia{dk, dv, s->n, s->G, s->Gpad, s->d_state};
+  grain_init_kernel<<<(s->G + kInitT - 1) / kInitT, kInitT, 0, s->stream>>>(ia);
+  return cudaGetLastError();
 }
 
 size_t grain_out_bytes(size_t n, uint64_t n_bits, int layout) {
@@ -637,9 +663,7 @@ MICKEY_API grain_streams *grain_init_streams(const void *keys, const void *ivs, 
     dv = s->d_inputs + n * 10;
   }
   if (ok) {
-    GrainInitArgs ia{dk, dv, n, s->G, s->Gpad, s->d_state};
-    grain_init_kernel<<<(s->G + kInitT - 1) / kInitT, kInitT, 0, s->stream>>>(ia);
-    ok = cudaGetLastError() == cudaSuccess;
+    ok = grain_init(s, dk, dv) == cudaSuccess;
   }
   if (!ok) {
     grain_release(s);
@@ -666,9 +690,7 @@ MICKEY_API int grain_reset_streams(grain_streams *s, const void *keys, const voi
     dk = s->d_inputs;
     dv = s->d_inputs + n * 10;
   }
-  GrainInitArgs ia{dk, dv, n, s->G, s->Gpad, s->d_state};
-  grain_init_kernel<<<(s->G + kInitT - 1) / kInitT, kInitT, 0, s->stream>>>(ia);
-  if (cudaGetLastError() != cudaSuccess) return grain_fail(MICKEY_E_CUDA, "grain init launch");
+  if (grain_init(s, dk, dv) != cudaSuccess) return grain_fail(MICKEY_E_CUDA, "grain init launch");
   s->pos = 0;
   return set_error(MICKEY_OK, "");
 }
@@ -680,6 +702,20 @@ MICKEY_API int grain_generate(grain_streams *s, uint64_t n_bits, void *out, int 
     return grain_fail(MICKEY_E_LAYOUT, "Grain takes the bitsliced or the bytes layout");
   if (layout == MICKEY_LAYOUT_BITSLICED_U32 && (reinterpret_cast<uintptr_t>(out) & 3u))
     return grain_fail(MICKEY_E_ARG, "bitsliced output must be 4-byte aligned");
+  // rows off the 16-byte grid cost the thread-per-group launch byte stores
+  // (1001 bits, 2^20 instances: 1196 us against 616), so those are packed at
+  // any size
+  const bool rows16 =
+      ((n_bits + 7) / 8) % 16 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+  const uint32_t per_sm = layout == MICKEY_LAYOUT_BITSLICED_U32 ? kGrainPackedBitslicedPerSm
+                          : rows16 ? kGrainPackedBytesPerSm : ~0u / uint32_t(s->sm_count);
+  if (grain_use_packed(s, per_sm)) {
+    const KeystreamArgs ka{s->d_state, s->G, s->Gpad, s->n, n_bits, out};
+    if (launch_grain_packed(ka, layout, s->stream) != cudaSuccess)
+      return grain_fail(MICKEY_E_CUDA, "grain keystream launch");
+    s->pos += n_bits;
+    return set_error(MICKEY_OK, "");
+  }
   const uint32_t tail = uint32_t(s->n & 31u);
   GrainArgs a{s->d_state, s->G, s->Gpad, s->n, n_bits, out, tail ? (1u << tail) - 1u : ~0u};
   const uint32_t W = (s->G + 31) / 32;

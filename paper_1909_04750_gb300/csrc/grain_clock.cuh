@@ -47,36 +47,46 @@ __device__ __forceinline__ uint32_t grain_z(const uint32_t (&b)[kG], uint32_t h0
 #undef B
 }
 
-// NFSR feedback s0 + g(b), the 23 terms in a tree (at most five dependent
-// steps), into slot R; s0 is the LFSR's oldest bit.
-template <int R, bool INIT>
-__device__ __forceinline__ void grain_nfsr(uint32_t (&b)[kG], uint32_t s0, uint32_t z) {
-#define B(i) b[(R + (i)) % kG]
-  const uint32_t p1 = B(63) & B(60);
-  const uint32_t p2 = B(37) & B(33);
-  const uint32_t p3 = B(15) & B(9);
-  const uint32_t q = B(60) & B(52);
-  const uint32_t r = B(52) & B(45);
-  const uint32_t p5 = and3(B(33), B(28), B(21));
-  const uint32_t p6 = and3(B(63), B(45), B(28));
-  const uint32_t l1 = xor3(B(62), B(60), B(52));
-  const uint32_t l2 = xor3(B(45), B(37), B(33));
-  const uint32_t l3 = xor3(B(28), B(21), B(14));
-  const uint32_t l4 = xor3(B(9), B(0), s0);
+// NFSR feedback s0 + g(b) of the tap words (+ z while initialising), the 23
+// terms in a tree (at most five dependent steps); s0 is the LFSR's oldest bit.
+template <bool INIT>
+__device__ __forceinline__ uint32_t grain_feedback(uint32_t s0, uint32_t z, uint32_t b0, uint32_t b9,
+                                                   uint32_t b14, uint32_t b15, uint32_t b21,
+                                                   uint32_t b28, uint32_t b33, uint32_t b37,
+                                                   uint32_t b45, uint32_t b52, uint32_t b60,
+                                                   uint32_t b62, uint32_t b63) {
+  const uint32_t p1 = b63 & b60;
+  const uint32_t p2 = b37 & b33;
+  const uint32_t p3 = b15 & b9;
+  const uint32_t q = b60 & b52;
+  const uint32_t r = b52 & b45;
+  const uint32_t p5 = and3(b33, b28, b21);
+  const uint32_t p6 = and3(b63, b45, b28);
+  const uint32_t l1 = xor3(b62, b60, b52);
+  const uint32_t l2 = xor3(b45, b37, b33);
+  const uint32_t l3 = xor3(b28, b21, b14);
+  const uint32_t l4 = xor3(b9, b0, s0);
   const uint32_t m1 = xor3(l1, l2, l3);                 // the linear terms ...
   const uint32_t m2 = xor3(l4, p1, p2);                 // ... s0, b63b60, b37b33
-  const uint32_t m3 = xand(p3, q, B(45));               // b15b9, b60b52b45
-  const uint32_t m4 = xand(p5, p6, B(9));               // b33b28b21, b63b45b28b9
-  const uint32_t t8 = and3(p1, B(21), B(15));           // b63b60b21b15
-  const uint32_t t9 = and3(p1, r, B(37));               // b63b60b52b45b37
-  const uint32_t t11 = and3(r, B(37), p5);              // b52b45b37b33b28b21
+  const uint32_t m3 = xand(p3, q, b45);                 // b15b9, b60b52b45
+  const uint32_t m4 = xand(p5, p6, b9);                 // b33b28b21, b63b45b28b9
+  const uint32_t t8 = and3(p1, b21, b15);               // b63b60b21b15
+  const uint32_t t9 = and3(p1, r, b37);                 // b63b60b52b45b37
+  const uint32_t t11 = and3(r, b37, p5);                // b52b45b37b33b28b21
   const uint32_t n1 = xor3(m1, m2, m3);
   const uint32_t n2 = xand(m4, q, p2);                  // b60b52b37b33
   const uint32_t n3 = xor3(t8, t9, t11);
   const uint32_t n4 = xand(n2, p5, p3);                 // b33b28b21b15b9
-  uint32_t nb = xor3(n1, n4, n3);
-  if (INIT) nb ^= z;
-  B(0) = nb;   // slot R: the oldest bit becomes the newest
+  const uint32_t nb = xor3(n1, n4, n3);
+  return INIT ? nb ^ z : nb;
+}
+
+// The same from the registers, into slot R: the oldest bit becomes the newest.
+template <int R, bool INIT>
+__device__ __forceinline__ void grain_nfsr(uint32_t (&b)[kG], uint32_t s0, uint32_t z) {
+#define B(i) b[(R + (i)) % kG]
+  B(0) = grain_feedback<INIT>(s0, z, B(0), B(9), B(14), B(15), B(21), B(28), B(33), B(37), B(45),
+                              B(52), B(60), B(62), B(63));
 #undef B
 }
 

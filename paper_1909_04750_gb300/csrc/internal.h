@@ -120,6 +120,13 @@ cudaError_t launch_ragged(const RaggedArgs &a, int layout, cudaStream_t st);
 // launch_keystream takes.
 cudaError_t launch_packed_keystream(const KeystreamArgs &a, int layout, cudaStream_t st);
 
+// Grain with one thread per instance (grain_packed.cu): the bitsliced or the
+// bytes layout, any n_bits and alignment that grain_generate takes; loading and
+// the 160 initialisation clocks.  State: s0..s79 then b0..b79, rows of Gpad words.
+cudaError_t launch_grain_packed(const KeystreamArgs &a, int layout, cudaStream_t st);
+cudaError_t launch_grain_packed_init(const uint8_t *keys, const uint8_t *ivs, uint64_t n,
+                                     uint32_t G, uint32_t Gpad, uint32_t *state, cudaStream_t st);
+
 // p == nullptr: grid mode (one thread per group); else persistent mode.
 // stage: row layouts stage this many tiles per row (grid: 2 or 4; persistent:
 // p->stage_tiles) and write whole chunks of 4 x stage bytes per row, used when

@@ -166,6 +166,44 @@ __device__ __forceinline__ uint32_t warp_transpose(uint32_t x, uint32_t lane) {
   return x;
 }
 
+// A lane's output row at o, written in whole words in memory order: four at a
+// time (16-byte stores) where `vec` says that output and pitch allow it, else
+// each word at the aligned addresses the row covers, put together from two
+// words of a row that starts off a word boundary (its first and last bytes go
+// singly).
+struct RowOut {
+  uint8_t *o;
+  bool vec, valid;
+  uint4 v;
+  __device__ __forceinline__ RowOut(uint8_t *row, bool vec16, bool lane_valid)
+      : o(row), vec(vec16), valid(lane_valid), v(make_uint4(0u, 0u, 0u, 0u)) {}
+  __device__ __forceinline__ void put(uint64_t t, uint32_t w) {   // word t = 0, 1, 2, ...
+    if (vec) {
+      v = make_uint4(v.y, v.z, v.w, w);
+      if ((t & 3) == 3 && valid) *reinterpret_cast<uint4 *>(o + 4 * (t - 3)) = v;
+      return;
+    }
+    const uint32_t a = uint32_t(reinterpret_cast<uintptr_t>(o)) & 3u;
+    const uint32_t x = __funnelshift_l(v.w, w, 8 * a);
+    v.w = w;
+    if (!valid) return;
+    if (t > 0 || a == 0)
+      *reinterpret_cast<uint32_t *>(o + 4 * t - a) = x;
+    else
+      for (uint32_t b = 0; b < 4 - a; ++b) o[b] = uint8_t(w >> (8 * b));
+  }
+  // After t whole words: the last one's bytes not yet written, then nbytes
+  // more of w.
+  __device__ __forceinline__ void finish(uint64_t t, int nbytes, uint32_t w) {
+    if (!valid) return;
+    const uint32_t a = uint32_t(reinterpret_cast<uintptr_t>(o)) & 3u;
+    uint8_t *p = o + 4 * t;
+    if (!vec && t > 0)
+      for (uint32_t b = 0; b < a; ++b) p[int(b) - int(a)] = uint8_t(v.w >> (32 - 8 * (a - b)));
+    for (int b = 0; b < nbytes; ++b) p[b] = uint8_t(w >> (8 * b));
+  }
+};
+
 // Group g's bitsliced state (word-major rows of P words, r0..r99 then
 // s0..s99) to the lanes' packed registers and back: lane j reads or writes
 // the row of bit j of each word, and the transpose turns rows into lanes.

@@ -144,3 +144,60 @@ def test_new_batch_plan_row_ends_at_any_tile(offset):
     for o, n in zip(b.offsets, nb):
         used[int(o):int(o) + (int(n) + 7) // 8] = True
     assert (host[~used] == 0xA5).all()
+
+
+def _grain(s):
+    from paper_1909_04750_gb300.grain import GrainStreams
+    return GrainStreams(torch.from_numpy(s.keys).cuda(), torch.from_numpy(s.ivs).cuda())
+
+
+# the 16-clock steps, the 160-clock body, tiles and 16-byte row stores, and what is left of each
+@pytest.mark.parametrize("n_bits", [1, 15, 16, 17, 31, 32, 33, 48, 128, 159, 160, 161, 176, 325,
+                                    1281])
+@pytest.mark.parametrize("n", [1, 33, 1000])
+def test_grain_two_calls_against_the_oracle(n, n_bits):
+    from oracle import grain as og
+    s = workloads.grain_streams(n, seed=21)
+    bits = np.unpackbits(og.batch_bytes(s.keys, s.ivs, n_bits + 67, threads=THREADS), axis=1,
+                         bitorder="little")
+    for layout in ("bytes", "bitsliced"):
+        st = _grain(s)
+        first, second = st.generate(n_bits, layout), st.generate(67, layout)
+        st.sync()
+        for got, lo, hi in ((first, 0, n_bits), (second, n_bits, n_bits + 67)):
+            want = np.packbits(bits[:, lo:hi], axis=1, bitorder="little")
+            a = got.cpu().numpy()
+            if layout == "bytes":
+                assert np.array_equal(a, want)
+            else:
+                assert np.array_equal(a.view(np.uint32), og.to_bitsliced(want, hi - lo))
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3, 4, 8])
+@pytest.mark.parametrize("n_bits", [5, 96, 256, 1001])
+def test_grain_output_at_any_alignment(n_bits, offset):
+    from oracle import grain as og
+    s = workloads.grain_streams(70, seed=22)
+    want = og.batch_bytes(s.keys, s.ivs, n_bits, threads=THREADS)
+    buf = torch.full((want.size + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+    st = _grain(s)
+    st.generate(n_bits, "bytes", out=buf[offset:])
+    st.sync()
+    got = buf.cpu().numpy()
+    assert np.array_equal(got[offset:offset + want.size].reshape(want.shape), want)
+    assert (got[:offset] == 0xA5).all() and (got[offset + want.size:] == 0xA5).all()
+
+
+@pytest.mark.parametrize("per_sm,layout", [(110, "bitsliced"), (128, "bytes"), (180, "bytes")])
+@pytest.mark.parametrize("extra", [0, 1])
+def test_grain_last_size_and_the_next_agree_with_a_thread_per_group(monkeypatch, per_sm, layout,
+                                                                    extra):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    s = workloads.grain_streams((per_sm * sms + extra) * 32 - 5, seed=23)
+    auto = _grain(s)
+    monkeypatch.setenv("MICKEY_GRAIN_QUEUE", "0")
+    grid = _grain(s)
+    for n_bits in (256, 333):
+        assert torch.equal(auto.generate(n_bits, layout), grid.generate(n_bits, layout))
+    k = 50_000
+    assert np.array_equal(auto.export_state()[:k], grid.export_state()[:k])
