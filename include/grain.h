@@ -19,17 +19,17 @@
  *           cause in mickey_last_error() / mickey_last_error_message().
  *  Streams  work is enqueued on the handle's CUDA stream; calls return once
  *           it is enqueued.
- *  Launch   with no more 32-group warp-groups than resident warps, one warp
- *           per warp-group clocks the whole call; with more, a persistent
- *           launch takes (warp-group, 1280-clock chunk) items from a queue,
- *           each chunk continuing from the state its predecessor published
- *           (a bounded wait: MICKEY_SPIN_LIMIT polls of about 256 ns, after
- *           which grain_sync reports MICKEY_E_TIMEOUT).  Handles with few
- *           groups (bitsliced up to 110 per SM, bytes up to 180 or any
+ *  Launch   per SM sub-partition a clock warp (a thread per group) paired
+ *           with an emission warp; with more 32-group warp-groups than clock
+ *           warps the groups x 32-clock tiles are cut into equal segments, a
+ *           segment continuing a warp-group from the state its predecessor
+ *           published (a bounded wait: MICKEY_SPIN_LIMIT polls of about 256
+ *           ns, after which grain_sync reports MICKEY_E_TIMEOUT).  Handles
+ *           with few groups (bitsliced up to 54 per SM, bytes up to 86 or any
  *           number when rows are not 16-byte aligned) run one thread per
  *           instance instead.  MICKEY_GRAIN_QUEUE, read when a handle is
- *           created: 1 forces the queue, 0 the warp per warp-group.  The bytes
- *           layout stages rows in tensor memory (one block of 8 warps per SM).
+ *           created: 1 forces segments that wait for their predecessors
+ *           whatever the number of groups, 0 the paired launch as above.
  */
 #ifndef GRAIN_H
 #define GRAIN_H

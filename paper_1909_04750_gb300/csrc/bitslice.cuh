@@ -148,6 +148,47 @@ __device__ __forceinline__ void transpose32(uint32_t (&a)[32]) {
   stage(std::integral_constant<int, 1>{}, 0x55555555u);
 }
 
+// a * b + c on the FMA pipe (written out: as C++ a product with a power of two
+// or a 0/1 value becomes shifts or logic operations, which the half-rate logic
+// pipe takes).
+__device__ __forceinline__ uint32_t mad32(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t d;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+
+// The same transpose in fewer logic-pipe operations: the 16- and 8-bit block
+// swaps are byte moves, one PRMT per word; the 4-, 2- and 1-bit swaps one
+// shift and one bit-select LOP3 per word, the left shifts as multiplies.
+__device__ __forceinline__ void transpose32_prmt(uint32_t (&a)[32]) {
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const uint32_t x = a[k], y = a[k + 16];
+    a[k] = __byte_perm(x, y, 0x3276);
+    a[k + 16] = __byte_perm(x, y, 0x1054);
+  }
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    if (k & 8) continue;
+    const uint32_t x = a[k], y = a[k + 8];
+    a[k] = __byte_perm(x, y, 0x3715);
+    a[k + 8] = __byte_perm(x, y, 0x2604);
+  }
+  auto stage = [&](auto jc, uint32_t m) {
+    constexpr int j = decltype(jc)::value;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      if (k & j) continue;
+      const uint32_t x = a[k], y = a[k + j];
+      a[k] = lop3<0xD8>(x, y >> j, m);               // (x & ~m) | ((y >> j) & m)
+      a[k + j] = lop3<0xD8>(y, mad32(x, 1u << j, 0u), m << j);
+    }
+  };
+  stage(std::integral_constant<int, 4>{}, 0x0F0F0F0Fu);
+  stage(std::integral_constant<int, 2>{}, 0x33333333u);
+  stage(std::integral_constant<int, 1>{}, 0x55555555u);
+}
+
 // Block swaps of the two-pass 32x32 transpose used to un-bitslice a tile
 // (see the keystream kernels).
 template <int J>

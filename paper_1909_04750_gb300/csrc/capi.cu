@@ -341,6 +341,7 @@ int launch_generate(mickey_streams *s, uint64_t bits, void *out, int layout) {
   pa.wait_epoch = s->test_unpublished ? (s->epoch | 0x80000000u) : s->epoch;
   pa.spin_limit = s->spin_limit;
   pa.err = s->d_err;
+  pa.tails_first = 0;
   CUDA_TRY(launch_keystream(ka, layout, unroll, stage, &pa, s->stream),
            "keystream persistent launch");
   return MICKEY_OK;

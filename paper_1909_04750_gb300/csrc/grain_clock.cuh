@@ -12,9 +12,7 @@ namespace mickey {
 namespace grainc {
 
 constexpr int kG = 80;               // register length
-constexpr int kGrainThreads = 64;    // groups per block (bitsliced layout)
-constexpr int kRing = 160;           // keystream words per thread in the ring
-constexpr int kRingStride = 32;      // each warp's ring is [word][lane]
+constexpr int kGrainThreads = 64;    // groups per block of the clock probe
 
 __device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) {
   return lop3<0x96>(a, b, c);
@@ -119,13 +117,82 @@ __device__ __forceinline__ uint32_t grain_clock(uint32_t (&s)[kG], uint32_t (&b)
   return z;
 }
 
-// 80 clocks (one full rotation); keystream word of clock c to zb[c * kRingStride].
-template <bool INIT>
-__device__ __forceinline__ void grain_body(uint32_t (&s)[kG], uint32_t (&b)[kG], uint32_t *zb) {
-  static_for<0, kG>([&](auto rc) {
-    constexpr int R = decltype(rc)::value;
-    const uint32_t z = grain_clock<R, INIT>(s, b);
-    if constexpr (!INIT) zb[R * kRingStride] = z;
+// U consecutive clocks from rotation R, operation by operation in turn (no
+// tap reaches the bits that U <= 16 clocks add): f(clock, z) takes each z.  The
+// interleaved order is what keeps the register need down: written clock by
+// clock, the compiler's schedule overlaps clocks until it spills.
+template <int R, int U, class F>
+__device__ __forceinline__ void grain_clocks(uint32_t (&s)[kG], uint32_t (&b)[kG], F &&f) {
+#define S(i) s[(R + u + (i)) % kG]
+#define B(i) b[(R + u + (i)) % kG]
+#define EACH(...) static_for<0, U>([&](auto uc) { constexpr int u = decltype(uc)::value; __VA_ARGS__; })
+  uint32_t p1[U], p2[U], p3[U], q[U], r[U], p5[U], p6[U], l1[U], l2[U], l3[U], l4[U], h0[U], h1[U];
+  EACH(p1[u] = B(63) & B(60));
+  EACH(p2[u] = B(37) & B(33));
+  EACH(p3[u] = B(15) & B(9));
+  EACH(q[u] = B(60) & B(52));
+  EACH(r[u] = B(52) & B(45));
+  EACH(p5[u] = and3(B(33), B(28), B(21)));
+  EACH(p6[u] = and3(B(63), B(45), B(28)));
+  EACH(l1[u] = xor3(B(62), B(60), B(52)));
+  EACH(l2[u] = xor3(B(45), B(37), B(33)));
+  EACH(l3[u] = xor3(B(28), B(21), B(14)));
+  EACH(l4[u] = xor3(B(9), B(0), S(0)));
+  EACH(l1[u] = xor3(l1[u], l2[u], l3[u]));                  // the linear terms ...
+  EACH(l4[u] = xor3(l4[u], p1[u], p2[u]));                  // ... s0, b63b60, b37b33
+  EACH(l2[u] = xand(p3[u], q[u], B(45)));                   // b15b9, b60b52b45
+  EACH(p6[u] = xand(p5[u], p6[u], B(9)));                   // b33b28b21, b63b45b28b9
+  EACH(l3[u] = and3(p1[u], B(21), B(15)));                  // b63b60b21b15
+  EACH(p1[u] = and3(p1[u], r[u], B(37)));                   // b63b60b52b45b37
+  EACH(r[u] = and3(r[u], B(37), p5[u]));                    // b52b45b37b33b28b21
+  EACH(p6[u] = xand(p6[u], q[u], p2[u]));                   // b60b52b37b33
+  EACH(l1[u] = xor3(l1[u], l4[u], l2[u]));
+  EACH(l3[u] = xor3(l3[u], p1[u], r[u]));
+  EACH(p6[u] = xand(p6[u], p5[u], p3[u]));                  // b33b28b21b15b9
+  EACH(l1[u] = xor3(l1[u], p6[u], l3[u]));
+  EACH(grain_h01(S(3), S(25), S(46), S(64), h0[u], h1[u]));
+  EACH(p2[u] = xor3(B(1), B(2), B(4)));
+  EACH(p3[u] = xor3(B(10), B(31), B(43)));
+  EACH(h0[u] = xand(h0[u], B(63), h1[u]));
+  EACH(p2[u] = xor3(p2[u], p3[u], B(56)));
+  EACH(f(uc, p2[u] ^ h0[u]));
+  EACH(q[u] = xor3(S(62), S(51), S(38)));
+  EACH(r[u] = xor3(S(23), S(13), S(0)));
+  EACH(S(0) = q[u] ^ r[u]);
+  EACH(B(0) = l1[u]);
+#undef EACH
+#undef S
+#undef B
+}
+
+// K clocks from rotation 0 (f(clock, z) takes each z), then the words back
+// to rotation 0: 80 - K moves per register.  K is kept small enough for the
+// instruction cache: 80 clocks need no moves, but their 2900 instructions
+// (46 KB) issued at 0.60 / 0.82 of the logic rate with one / two warps per SM
+// sub-partition, 40 clocks (23 KB) at 0.87 / 0.90, 20 at 0.83 / 0.90 (clocks
+// with ring stores, GB300).
+template <int K, bool INIT, class F>
+__device__ __forceinline__ void grain_body(uint32_t (&s)[kG], uint32_t (&b)[kG], F &&f) {
+  if constexpr (INIT) {
+    static_for<0, K>([&](auto rc) { grain_clock<decltype(rc)::value, true>(s, b); });
+  } else {
+    static_for<0, K / 4>([&](auto kc) {
+      constexpr int R = 4 * decltype(kc)::value;
+      grain_clocks<R, 4>(s, b, [&](auto uc, uint32_t z) {
+        f(std::integral_constant<int, R + decltype(uc)::value>{}, z);
+      });
+    });
+  }
+  uint32_t ts[kG], tb[kG];
+  static_for<0, kG>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    ts[i] = s[(i + K) % kG];
+    tb[i] = b[(i + K) % kG];
+  });
+  static_for<0, kG>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    s[i] = ts[i];
+    b[i] = tb[i];
   });
 }
 

@@ -101,6 +101,8 @@ struct PersistArgs {
                         // MICKEY_TEST_UNPUBLISHED test hook, to make the wait run out)
   uint32_t spin_limit;  // bounded wait of a tail piece (iterations of ~256 ns)
   int *err;
+  uint32_t tails_first; // 1: each segment runs its tail piece first, so that every hand-off
+                        // is waited for (a test's order; 0: heads first, hardly any wait)
 };
 
 // Ragged generation on a handle (ragged.cu): stream i continues by
@@ -124,6 +126,10 @@ cudaError_t launch_packed_keystream(const KeystreamArgs &a, int layout, cudaStre
 // bytes layout, any n_bits and alignment that grain_generate takes; loading and
 // the 160 initialisation clocks.  State: s0..s79 then b0..b79, rows of Gpad words.
 cudaError_t launch_grain_packed(const KeystreamArgs &a, int layout, cudaStream_t st);
+// Grain with clock warps paired with emission warps (grain_ws.cu), any
+// n_bits and alignment; `p` as for the paired keystream launch.
+cudaError_t launch_grain_ws(const KeystreamArgs &a, int layout, const PersistArgs &p,
+                            cudaStream_t st);
 cudaError_t launch_grain_packed_init(const uint8_t *keys, const uint8_t *ivs, uint64_t n,
                                      uint32_t G, uint32_t Gpad, uint32_t *state, cudaStream_t st);
 

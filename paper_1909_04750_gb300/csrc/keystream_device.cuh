@@ -9,6 +9,15 @@
 
 namespace mickey {
 
+// Internal layout of the emission code: byte rows whose first keystream bit is
+// the least significant bit (Grain).  The tile's rows come in reverse order
+// (row i = clock 31 - i), so the transposed word is in memory order as it is.
+constexpr int kLayoutBytesLsb = 16;
+template <int LAYOUT>
+__host__ __device__ constexpr bool byte_rows() {
+  return LAYOUT == MICKEY_LAYOUT_BYTES || LAYOUT == kLayoutBytesLsb;
+}
+
 struct EmitCtx {
   uint32_t lane_mask;  // valid lanes of this group (last group may be partial)
   bool vec_ok;         // 16-byte vector stores allowed (bitsliced layout)
@@ -50,7 +59,7 @@ __device__ __forceinline__ void store_row_word(uint8_t *tile, uint32_t pitch,
                                                uint64_t f32_off, int l, int nb,
                                                const EmitCtx &e, uint32_t word) {
   uint8_t *o = tile + uint64_t(uint32_t(l) * pitch);
-  if constexpr (LAYOUT == MICKEY_LAYOUT_BYTES) {
+  if constexpr (byte_rows<LAYOUT>()) {
     if (nb == 32 && e.word_ok) {
       *reinterpret_cast<uint32_t *>(o) = word;
     } else {
@@ -85,6 +94,21 @@ __device__ __forceinline__ void emit_slice(uint32_t *z, uint32_t *rb, const Keys
       v.z = z[(4 * j + 2) * kKsThreads] & e.lane_mask;
       v.w = z[(4 * j + 3) * kKsThreads] & e.lane_mask;
       reinterpret_cast<uint4 *>(o)[j] = v;
+    } else if (nb == 32) {
+      // a row off the 16-byte grid: the tile's words from its first 16-byte
+      // boundary on (word h) in vectors, the others singly
+      const int h = int((4u - ((reinterpret_cast<uintptr_t>(o) >> 2) & 3u)) & 3u), c = h + 4 * j;
+      for (int k = 0; j == 0 && k < h; ++k) o[k] = z[k * kKsThreads] & e.lane_mask;
+      if (c + 4 <= 32) {
+        uint4 v;
+        v.x = z[(c + 0) * kKsThreads] & e.lane_mask;
+        v.y = z[(c + 1) * kKsThreads] & e.lane_mask;
+        v.z = z[(c + 2) * kKsThreads] & e.lane_mask;
+        v.w = z[(c + 3) * kKsThreads] & e.lane_mask;
+        *reinterpret_cast<uint4 *>(o + c) = v;
+      } else {
+        for (int k = c; k < 32; ++k) o[k] = z[k * kKsThreads] & e.lane_mask;
+      }
     } else {
       for (int c = 4 * j; c < 4 * j + 4 && c < nb; ++c) o[c] = z[c * kKsThreads] & e.lane_mask;
     }
@@ -101,8 +125,8 @@ __device__ __forceinline__ void emit_slice(uint32_t *z, uint32_t *rb, const Keys
 #pragma unroll
     for (int k = 0; k < 8; ++k) z[(8 * j + k) * kKsThreads] = v[k];
   } else {
-    const uint32_t pitch = LAYOUT == MICKEY_LAYOUT_BYTES ? uint32_t((a.n_bits + 7) >> 3)
-                                                         : uint32_t(a.n_bits >> 3);
+    const uint32_t pitch = byte_rows<LAYOUT>() ? uint32_t((a.n_bits + 7) >> 3)
+                                               : uint32_t(a.n_bits >> 3);
     uint8_t *tile = static_cast<uint8_t *>(a.out) + 32ull * g * pitch + (t0 >> 3);
     const uint64_t f32_off = uint64_t(pitch) * a.n;  // float block follows
 #pragma unroll

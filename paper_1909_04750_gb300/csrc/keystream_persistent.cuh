@@ -38,6 +38,7 @@ __device__ __forceinline__ bool segment_piece(const PersistArgs &p, uint64_t NT,
   const uint64_t full_n = full_end > full_lo ? full_end - full_lo : 0;
   const uint64_t n_pieces = (has_head ? 1 : 0) + full_n + (has_tail ? 1 : 0);
   if (k >= n_pieces) return false;
+  if (p.tails_first) k = uint32_t(n_pieces) - 1 - k;
   const uint64_t kk = k - (has_head ? 1 : 0);
   const uint64_t ww = (has_head && k == 0) ? w_last : (kk < full_n ? full_lo + kk : w_first);
   w = uint32_t(ww);

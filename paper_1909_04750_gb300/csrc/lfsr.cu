@@ -191,38 +191,6 @@ __global__ void __launch_bounds__(TB)
 constexpr int kCrcThreads = 64;
 constexpr int kCrcChunk = 16;
 
-// The 32 x 32 bit transpose of transpose32 (same result) in fewer ops:
-// the 16- and 8-bit block swaps are byte moves, one PRMT per word; the 4-,
-// 2- and 1-bit swaps are one shift and one bit-select LOP3 per word.
-__device__ __forceinline__ void transpose32_prmt(uint32_t (&a)[32]) {
-#pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const uint32_t x = a[k], y = a[k + 16];
-    a[k] = __byte_perm(x, y, 0x3276);
-    a[k + 16] = __byte_perm(x, y, 0x1054);
-  }
-#pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    if (k & 8) continue;
-    const uint32_t x = a[k], y = a[k + 8];
-    a[k] = __byte_perm(x, y, 0x3715);
-    a[k + 8] = __byte_perm(x, y, 0x2604);
-  }
-  auto stage = [&](auto jc, uint32_t m) {
-    constexpr int j = decltype(jc)::value;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      if (k & j) continue;
-      const uint32_t x = a[k], y = a[k + j];
-      a[k] = lop3<0xD8>(x, y >> j, m);               // (x & ~m) | ((y >> j) & m)
-      a[k + j] = lop3<0xD8>(y, x << j, m << j);
-    }
-  };
-  stage(std::integral_constant<int, 4>{}, 0x0F0F0F0Fu);
-  stage(std::integral_constant<int, 2>{}, 0x33333333u);
-  stage(std::integral_constant<int, 1>{}, 0x55555555u);
-}
-
 // Message m0 + l's CRC: bit k from s[k], lane l; then the final XOR.
 __device__ __forceinline__ void store_crcs(const uint32_t (&s)[8], size_t m0, size_t n,
                                            uint32_t xorout, uint8_t *crc) {

@@ -72,14 +72,6 @@ constexpr PackedMasks make_packed_masks() {
 }
 constexpr PackedMasks kPackedMasks = make_packed_masks();
 
-// a * b + c on the FMA pipe (written out: as C++ the products with 0/1 become
-// logic operations).
-__device__ __forceinline__ uint32_t mad32(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-  return d;
-}
-
 // One CLOCK_KG of the thread's instance; MIX as in clock_kg, `in` 0 or 1.
 template <bool MIX>
 __device__ __forceinline__ void clock_packed(Packed &q, uint32_t in) {

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(128, 1)
 
 // The bare Grain clock: 64 threads per block, one 32-lane group per thread,
 // `bodies` x 80 clocks from an arbitrary state; STORE writes each clock's
-// keystream word to shared memory (as the keystream kernel's ring does),
+// keystream word to shared memory (as the keystream kernel's tile buffers take it),
 // otherwise the words are folded into an accumulator.
 template <bool STORE>
 __global__ void __launch_bounds__(mickey::grainc::kGrainThreads)
@@ -102,14 +102,14 @@ __global__ void __launch_bounds__(mickey::grainc::kGrainThreads)
   uint32_t acc = 0;
 #pragma unroll 1
   for (int k = 0; k < bodies; ++k) {
-    if constexpr (STORE) {
-      grain_body<false>(s, b, zb + (threadIdx.x >> 5) * (kG * kRingStride) + (threadIdx.x & 31));
-    } else {
-      mickey::static_for<0, kG>([&](auto rc) {
-        constexpr int R = decltype(rc)::value;
-        acc ^= grain_clock<R, false>(s, b);
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h)
+      grain_body<40, false>(s, b, [&](auto rc, uint32_t z) {
+        if constexpr (STORE)
+          zb[(40 * h + decltype(rc)::value) * kGrainThreads + threadIdx.x] = z;
+        else
+          acc ^= z;
       });
-    }
   }
   __syncthreads();
   const long long t1 = clock64();

@@ -188,7 +188,7 @@ def test_grain_output_at_any_alignment(n_bits, offset):
     assert (got[:offset] == 0xA5).all() and (got[offset + want.size:] == 0xA5).all()
 
 
-@pytest.mark.parametrize("per_sm,layout", [(110, "bitsliced"), (128, "bytes"), (180, "bytes")])
+@pytest.mark.parametrize("per_sm,layout", [(54, "bitsliced"), (86, "bytes"), (128, "bytes")])
 @pytest.mark.parametrize("extra", [0, 1])
 def test_grain_last_size_and_the_next_agree_with_a_thread_per_group(monkeypatch, per_sm, layout,
                                                                     extra):
@@ -201,3 +201,36 @@ def test_grain_last_size_and_the_next_agree_with_a_thread_per_group(monkeypatch,
         assert torch.equal(auto.generate(n_bits, layout), grid.generate(n_bits, layout))
     k = 50_000
     assert np.array_equal(auto.export_state()[:k], grid.export_state()[:k])
+
+
+@pytest.mark.parametrize("queue", ["0", "1"])
+@pytest.mark.parametrize("n_bits", [32, 33, 128, 384, 256 * 3, 640, 2048 + 128, 1000])
+def test_grain_paired_launch_tiles_and_blocks(monkeypatch, n_bits, queue):
+    # row blocks of 8 tiles that end early, the ring of 12, segments that start
+    # and end inside a block (queue 1: three warp-groups on two chains), twice
+    from oracle import grain as og
+    monkeypatch.setenv("MICKEY_GRAIN_QUEUE", queue)
+    s = workloads.grain_streams(2 * 1024 + 70, seed=24)
+    bits = np.unpackbits(og.batch_bytes(s.keys, s.ivs, 2 * n_bits, threads=THREADS), axis=1,
+                         bitorder="little")
+    for layout in ("bytes", "bitsliced"):
+        st = _grain(s)
+        for k in range(2):
+            a = st.generate(n_bits, layout).cpu().numpy()
+            st.sync()
+            want = np.packbits(bits[:, k * n_bits:(k + 1) * n_bits], axis=1, bitorder="little")
+            if layout == "bytes":
+                assert np.array_equal(a, want)
+            else:
+                assert np.array_equal(a.view(np.uint32), og.to_bitsliced(want, n_bits))
+
+
+@pytest.mark.parametrize("n_bits", [1001, 1002, 67])
+def test_bitsliced_rows_off_the_16_byte_grid(monkeypatch, n_bits):
+    # the paired MICKEY launch stores a tile's words in vectors from the first
+    # 16-byte boundary on
+    monkeypatch.setenv("MICKEY_MODE", "persistent")
+    s = _mixed(300)
+    want = oracle.batch_bytes(s.keys, s.ivs, s.iv_lens, n_bits, threads=THREADS)
+    got = _streams(s).generate(n_bits, "bitsliced").cpu().numpy().view(np.uint32)
+    assert np.array_equal(got, oracle.to_bitsliced(want, n_bits))
