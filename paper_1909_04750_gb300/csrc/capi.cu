@@ -293,6 +293,17 @@ bool use_persistent(const mickey_streams *s, int mode) {
   return mode != MICKEY_MODE_GRID && W >= slots;
 }
 
+// The flags and the epoch that the segments of one launch hand states on with.
+void set_hand_off(mickey_streams *s, PersistArgs &pa) {
+  pa.flags = s->d_flags;
+  s->epoch = s->epoch % 0x7fffffffu + 1;   // 1 .. 2^31 - 1 (0 is the flags' initial value)
+  pa.epoch = s->epoch;
+  pa.wait_epoch = s->test_unpublished ? (s->epoch | 0x80000000u) : s->epoch;
+  pa.spin_limit = s->spin_limit;
+  pa.err = s->d_err;
+  pa.tails_first = 0;
+}
+
 // One keystream launch of `bits` clocks into a device buffer.
 //   AUTO, few groups          one thread per instance
 //   GRID                      one thread per group, clocking and emitting
@@ -335,13 +346,7 @@ int launch_generate(mickey_streams *s, uint64_t bits, void *out, int layout) {
     pa.cooperative = 0;
     pa.L = NT;
   }
-  pa.flags = s->d_flags;
-  s->epoch = s->epoch % 0x7fffffffu + 1;   // 1 .. 2^31 - 1 (0 is the flags' initial value)
-  pa.epoch = s->epoch;
-  pa.wait_epoch = s->test_unpublished ? (s->epoch | 0x80000000u) : s->epoch;
-  pa.spin_limit = s->spin_limit;
-  pa.err = s->d_err;
-  pa.tails_first = 0;
+  set_hand_off(s, pa);
   CUDA_TRY(launch_keystream(ka, layout, unroll, stage, &pa, s->stream),
            "keystream persistent launch");
   return MICKEY_OK;
@@ -514,7 +519,8 @@ int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
   // The lengths and offsets reach the kernel through one of two pinned
   // buffers (so that the copy is a DMA and the next call can fill the other
   // buffer while this one is in flight) and one device buffer.
-  const size_t words = n + n_off;
+  // ... then the prefix sums of the warp-groups' blocks
+  const size_t W = (G + 31) / 32, words = n + n_off + W + 1;
   if (s->ragged_words < words) {
     if (s->ev_ragged) CUDA_TRY(cudaEventSynchronize(s->ev_ragged), "sync");
     for (int k = 0; k < 2; ++k) {
@@ -543,6 +549,15 @@ int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
     std::copy(out_offsets, out_offsets + n_off, h + n);
   else
     ragged_packed(n, n_bits, layout, h + n);
+  uint64_t *blocks = h + n + n_off, longest = 0;
+  blocks[0] = 0;
+  for (size_t w = 0; w < W; ++w) {
+    uint64_t c = 0;
+    for (size_t i = 1024 * w; i < std::min(n, 1024 * w + 1024); ++i) c = std::max(c, n_bits[i]);
+    c = (c + kRaggedBlockBits - 1) / kRaggedBlockBits;
+    blocks[w + 1] = blocks[w] + c;
+    longest = std::max(longest, c);
+  }
   // the previous ragged launch (perhaps on another stream) has read d_ragged
   CUDA_TRY(cudaStreamWaitEvent(s->stream, s->ev_ragged, 0), "wait");
   CUDA_TRY(cudaMemcpyAsync(s->d_ragged, h, words * 8, cudaMemcpyHostToDevice, s->stream),
@@ -550,8 +565,17 @@ int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
   CUDA_TRY(cudaEventRecord(s->ev_h2d[kb], s->stream), "record");
   s->ragged_flip = kb ^ 1;
   RaggedArgs ra{s->d_state, s->G, s->Gpad, n, s->d_ragged, s->d_ragged + n,
-                static_cast<uint8_t *>(out)};
-  CUDA_TRY(launch_ragged(ra, layout, s->stream), "ragged_kernel launch");
+                static_cast<uint8_t *>(out), s->d_ragged + n + n_off};
+  const auto &c = s->cfg[layout];
+  const bool packed = (c.set ? c.mode : s->mode) == MICKEY_MODE_AUTO && use_packed(s);
+  const uint64_t slots = std::min<uint64_t>(W, 4ull * uint32_t(s->persist_blocks));
+  PersistArgs pa{};
+  pa.blocks = uint32_t((slots + 3) / 4);
+  pa.cooperative = slots < W;
+  pa.W = uint32_t(W);
+  pa.L = std::max(longest, (blocks[W] + slots - 1) / slots);
+  set_hand_off(s, pa);
+  CUDA_TRY(launch_ragged(ra, layout, packed ? nullptr : &pa, s->stream), "ragged launch");
   CUDA_TRY(cudaEventRecord(s->ev_ragged, s->stream), "record");
   for (size_t i = 0; i < n; ++i) {
     s->pos[i] += n_bits[i];

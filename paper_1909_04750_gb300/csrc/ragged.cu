@@ -1,100 +1,83 @@
-// Ragged keystream generation on a streams handle: every stream continues
-// by its own number of bits in one launch (the instance-per-lane design of
+// Ragged keystream generation on a streams handle: every stream continues by
+// its own number of bits in one call (the instance-per-lane design of
 // Sec. IV-D with uneven lengths).
 //
-// One thread owns one 32-lane group, as in the keystream kernels: the
-// group's 200 state words stay in registers and the group is clocked as
-// many times as its longest lane needs.  Two things make the lanes' lengths
-// differ without a per-clock cost:
-//   * the keystream word of a clock is taken as (r0 ^ s0) & alive, one LOP3
-//     like the plain XOR, where `alive` holds the lanes whose length has not
-//     been reached; the bits of finished lanes are zero, so a row store only
-//     has to stop at the row's last byte;
-//   * a lane's state must be the one after exactly its own number of clocks.
-//     When the group starts, the bits of every lane with a length above 0
-//     are cleared in the state in HBM (unless all lanes share one length);
-//     at each distinct end point E of the group (at most 32) the current
-//     words, masked to the lanes ending at E, are OR-ed in (one fire-and-
-//     forget atomic per word, so the clock loop does not wait for memory),
-//     or stored outright when those lanes are all the group's lanes.  Lanes
-//     asked for 0 bits are never touched.
-// The clock loop takes one clock per iteration, so that the write-back code
-// exists once: a thread that takes it holds up its warp, and unrolled copies
-// of it were instruction-cache misses each time.  The values the next clock
-// reads besides neighbouring bits (control bit, feedback bits) are computed
-// inside the iteration, so the loop's back edge does not wait on them.  An
-// end point is found from a per-tile mask of the clocks at which some lane
-// ends; the lanes ending there are looked up only then.  Every fourth clock
-// emits one eighth of the previous tile (as the keystream kernels do).  The
-// last tile is clocked in full: past the longest lane every lane has been
-// written back and the extra keystream bits are zero and not stored.
-#include "bitslice.cuh"
-#include "internal.h"
-#include "../../include/mickey.h"
+// Few groups (ragged_packed_kernel): one thread per instance (packed.cuh).  A
+// thread clocks its own stream as often as it needs and is done.
+//
+// Many groups (ragged_ws_kernel): one thread per 32-lane group, clock warps
+// paired with emission warps as in the keystream launch
+// (keystream_persistent.cuh); a group is clocked as often as its longest lane
+// needs.  What differs from equal lengths:
+//   * The work line of warp-groups x blocks of 128 clocks has as many blocks
+//     per warp-group as its longest lane; segments are cut on the prefix sums,
+//     each at least as long as the longest warp-group, so that a warp-group
+//     spans two at most.
+//   * A lane's state must be the one after exactly its own number of clocks.
+//     The clock loop has no test per clock: before every block the lanes that
+//     end within its 128 clocks are merged into the state in HBM
+//     (their bits were cleared there when the piece started, so one
+//     fire-and-forget OR per word sets them), and ragged_rest_kernel runs
+//     each lane's remaining 0 .. 127 clocks with a thread per instance.
+//   * The emission warp knows where each row ends: whole words go out at the
+//     aligned addresses a row covers (rows start at any byte), the last ones
+//     byte by byte.
+// Bound by the logic pipe: the clocks of the longest lanes (0.76 of the clocked
+// bits are output below), then the emission warp's share of it.  Measured, 2^20
+// streams, lengths uniform in [2^13, 2^14], bytes at the packed offsets, call
+// by call: 21.9 -> 11.7 ms (1105 Gbit/s); before, one warp clocked, tested each
+// clock for ends and emitted with byte stores.
+#include "keystream_persistent.cuh"
+#include "packed.cuh"
 
 namespace mickey {
 namespace {
 
-constexpr int kRaggedThreads = 64;
+// Tiles per block.  States are handed on at block boundaries only: a lane that
+// has been merged then has no output left in the next segment.
+constexpr uint32_t kSnapTiles = kRaggedBlockBits / 32;
 
-// Per-thread view of the group's lanes in shared memory: lane l's length at
-// bits[l * kRaggedThreads] and its output row's address at row[l * kRaggedThreads]
-// (columns of one thread, so a warp's accesses are conflict-free).
+// ------------------------------------------------------- one thread per group
+
+// Shared memory of a block after the two tile buffers, all [lane][thread]:
+// a row's address, the previous tile's word, the tiles that hold the lane's
+// bits, and the tile before which its state is merged (~0: no bits asked for).
 struct LaneTab {
-  const uint64_t *bits;
-  uint8_t *const *row;
+  uint64_t *row;
+  uint32_t *carry, *tiles, *snap;
 };
+constexpr size_t kRaggedSmem = 4 * kTileBufWords + size_t(32) * kKsThreads * (8 + 4 + 4 + 4);
 
-// Bit k set when some lane's length is t0 + k + 1 (its last clock is clock
-// k of the tile starting at call clock t0).
-__device__ __forceinline__ uint32_t tile_ends(const LaneTab &lt, int lanes, uint64_t t0) {
-  uint32_t e = 0;
-  for (int l = 0; l < lanes; ++l) {
-    const uint64_t d = lt.bits[l * kRaggedThreads] - t0 - 1;   // wraps for lengths <= t0
-    if (d < 32) e |= 1u << d;
-  }
-  return e;
+__device__ __forceinline__ LaneTab lane_tab(uint32_t *zs, uint32_t t) {
+  uint64_t *row = reinterpret_cast<uint64_t *>(zs + kTileBufWords);
+  uint32_t *w = reinterpret_cast<uint32_t *>(row + 32 * kKsThreads);
+  return LaneTab{row + t, w + t, w + 32 * kKsThreads + t, w + 64 * kKsThreads + t};
 }
 
-// The lanes whose length is exactly E.
-__device__ __forceinline__ uint32_t lanes_ending(const LaneTab &lt, int lanes, uint64_t E) {
+// The lanes for which f(snap tile) holds.
+template <class F>
+__device__ __forceinline__ uint32_t lanes_where(const uint32_t *snap, F f) {
   uint32_t m = 0;
-  for (int l = 0; l < lanes; ++l) m |= (lt.bits[l * kRaggedThreads] == E ? 1u : 0u) << l;
+#pragma unroll 8
+  for (int l = 0; l < 32; ++l) m |= (f(snap[l * kKsThreads]) ? 1u : 0u) << l;
   return m;
 }
 
-// True when every lane has length C (then the one end point writes the
-// whole group back with plain stores).
-__device__ __forceinline__ bool same_end(const LaneTab &lt, int lanes, uint64_t C) {
-  for (int l = 0; l < lanes; ++l)
-    if (lt.bits[l * kRaggedThreads] != C) return false;
-  return true;
-}
-
-// Truth table of (a ^ b) & c (operands a, b, c = 0xF0, 0xCC, 0xAA).
-constexpr uint32_t kXorAnd = ((0xF0u ^ 0xCCu) & 0xAAu) & 0xFFu;              // 0x28
-
-// Merge the lanes in `m` of the current state into the state in HBM
-// (`pad`: lanes past the last instance, whose bits nothing reads).  The bits
-// of every lane with a length above 0 were cleared in HBM when the group
-// started, so setting the ones is enough.  The base address and stride
-// pass through an opaque move, so that the 200 word addresses are formed
-// here, when the branch is taken, and are not held live across the clock
-// loop (which spilled).
-__device__ __forceinline__ void snapshot(uint32_t *st0, size_t P0, const uint32_t (&r)[kReg],
-                                         const uint32_t (&s)[kReg], uint32_t m, uint32_t pad) {
+// The address of the group's state and the row pitch through an opaque move,
+// so that the 200 word addresses are formed where they are used and are not
+// held live across the clock loop (which spilled).
+__device__ __forceinline__ uint32_t *opaque(uint32_t *st0, size_t P0, size_t &P) {
   uint32_t *st;
-  size_t P;
   asm volatile("mov.b64 %0, %1;" : "=l"(st) : "l"(st0));
   asm volatile("mov.b64 %0, %1;" : "=l"(P) : "l"(P0));
-  if ((m | pad) == ~0u) {
-#pragma unroll
-    for (int i = 0; i < kReg; ++i) {
-      st[size_t(i) * P] = r[i];
-      st[size_t(kReg + i) * P] = s[i];
-    }
-    return;
-  }
+  return st;
+}
+
+// OR the lanes in `m` of the current state into the state in HBM.
+__device__ __forceinline__ void merge_lanes(uint32_t *st0, size_t P0, const uint32_t (&r)[kReg],
+                                            const uint32_t (&s)[kReg], uint32_t m) {
+  size_t P;
+  uint32_t *st = opaque(st0, P0, P);
 #pragma unroll
   for (int i = 0; i < kReg; ++i) {
     atomicOr(st + size_t(i) * P, r[i] & m);
@@ -102,179 +85,360 @@ __device__ __forceinline__ void snapshot(uint32_t *st0, size_t P0, const uint32_
   }
 }
 
-// Store the finished word w of lane l (z_{t0} first; memory byte order for
-// the bytes layout, big-endian for u32) of the tile starting at call clock
-// t0, up to the lane's last byte.
+// Row of the tile buffer that takes clock c's word, such that the transposed
+// word of a lane is in memory order (bytes) or big-endian (u32).
 template <int LAYOUT>
-__device__ __forceinline__ void store_lane(const LaneTab &lt, int l, uint64_t t0, uint32_t w) {
-  const uint64_t bits = lt.bits[l * kRaggedThreads];
-  if (t0 >= bits) return;
-  uint8_t *o = lt.row[l * kRaggedThreads] + (t0 >> 3);
-  const uint64_t left = bits - t0;
-  if (left >= 32 && (reinterpret_cast<uintptr_t>(o) & 3u) == 0) {
-    *reinterpret_cast<uint32_t *>(o) = w;
-    return;
-  }
-  // bytes layout only: a last partial word or an unaligned row
-  const int nbytes = left >= 32 ? 4 : int((left + 7) >> 3);
-  for (int b = 0; b < nbytes; ++b) o[b] = uint8_t(w >> (8 * b));
-}
-
-// One eighth of a tile's emission (slices must run in order 0..7).
-//   bitsliced  slice j stores words 4j..4j+3 of the group's row;
-//   row-major  the two-pass in-place transpose of the keystream kernels:
-//              slices 0-3 swap blocks of size 4, 2, 1; slices 4-7 swap blocks
-//              of size 16 and 8 and store.
-template <int LAYOUT>
-__device__ __forceinline__ void ragged_slice(uint32_t *z, const LaneTab &lt, uint8_t *grow,
-                                             int lanes, uint64_t t0, int cnt, uint64_t C,
-                                             int j) {
-  if constexpr (LAYOUT == MICKEY_LAYOUT_BITSLICED_U32) {
-    uint32_t *o = reinterpret_cast<uint32_t *>(grow) + t0;
-    if (cnt == 32 && (reinterpret_cast<uintptr_t>(o) & 15u) == 0) {
-      uint4 v;
-      v.x = z[(4 * j + 0) * kRaggedThreads];
-      v.y = z[(4 * j + 1) * kRaggedThreads];
-      v.z = z[(4 * j + 2) * kRaggedThreads];
-      v.w = z[(4 * j + 3) * kRaggedThreads];
-      reinterpret_cast<uint4 *>(o)[j] = v;
-    } else {
-      for (int c = 4 * j; c < 4 * j + 4 && uint64_t(c) < C - t0 && c < cnt; ++c)
-        o[c] = z[c * kRaggedThreads];
-    }
-  } else if (j < 4) {
-    uint32_t v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = z[(8 * j + k) * kRaggedThreads];
-    swap_bits<4>(v[0], v[4]); swap_bits<4>(v[1], v[5]);
-    swap_bits<4>(v[2], v[6]); swap_bits<4>(v[3], v[7]);
-    swap_bits<2>(v[0], v[2]); swap_bits<2>(v[1], v[3]);
-    swap_bits<2>(v[4], v[6]); swap_bits<2>(v[5], v[7]);
-    swap_bits<1>(v[0], v[1]); swap_bits<1>(v[2], v[3]);
-    swap_bits<1>(v[4], v[5]); swap_bits<1>(v[6], v[7]);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) z[(8 * j + k) * kRaggedThreads] = v[k];
-  } else {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = 2 * (j - 4) + h;
-      uint32_t v[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) v[q] = z[(k + 8 * q) * kRaggedThreads];
-      swap_halves(v[0], v[2]);
-      swap_halves(v[1], v[3]);
-      swap_bytes<LAYOUT == MICKEY_LAYOUT_BYTES>(v[0], v[1]);
-      swap_bytes<LAYOUT == MICKEY_LAYOUT_BYTES>(v[2], v[3]);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int l = 31 - k - 8 * q;   // row k + 8q of the transposed tile
-        if (l < lanes) store_lane<LAYOUT>(lt, l, t0, v[q]);
-      }
-    }
-  }
+__device__ __forceinline__ int clock_row(int c) {
+  return LAYOUT == MICKEY_LAYOUT_BYTES ? 24 - (c & ~7) + (c & 7) : c;
 }
 
 template <int LAYOUT>
-__device__ __forceinline__ void ragged_tile(uint32_t *z, const LaneTab &lt, uint8_t *grow,
-                                            int lanes, uint64_t t0, int cnt, uint64_t C) {
-#pragma unroll 1
-  for (int j = 0; j < 8; ++j) ragged_slice<LAYOUT>(z, lt, grow, lanes, t0, cnt, C, j);
-}
-
-// In-tile index of the clock after which the lanes ending at `next` are done
-// (next > t0), or 64 when that end point lies beyond the tile.
-__device__ __forceinline__ int end_in_tile(uint64_t next, uint64_t t0) {
-  return next - t0 - 1 < 32 ? int(next - t0 - 1) : 64;
-}
-
-// Shared memory of a block: two tile buffers (32 words per thread), then the
-// lane table: lengths and row addresses, 32 of each per thread.
-constexpr size_t kRaggedSmem = (2 * 32 * 4 + 32 * 8 + 32 * 8) * size_t(kRaggedThreads);
-
-template <int LAYOUT>
-__global__ void __launch_bounds__(kRaggedThreads) ragged_kernel(RaggedArgs a) {
-  extern __shared__ __align__(16) uint32_t zs[];
-  uint64_t *tab = reinterpret_cast<uint64_t *>(zs + 2 * 32 * kRaggedThreads);
-  const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= a.G) return;
-  const uint64_t base = uint64_t(g) * 32;
-  const int lanes = a.n - base >= 32 ? 32 : int(a.n - base);
-  const uint32_t pad = lanes < 32 ? ~0u << lanes : 0u;
-  LaneTab lt{tab + threadIdx.x, reinterpret_cast<uint8_t *const *>(tab + 32 * kRaggedThreads +
-                                                                    threadIdx.x)};
-  uint64_t C = 0;
-  uint32_t alive = 0;
-  for (int l = 0; l < lanes; ++l) {
-    const uint64_t b = a.n_bits[base + l];
-    tab[l * kRaggedThreads + threadIdx.x] = b;
-    if (LAYOUT != MICKEY_LAYOUT_BITSLICED_U32)
-      tab[(32 + l) * kRaggedThreads + threadIdx.x] =
-          reinterpret_cast<uint64_t>(a.out + a.offsets[base + l]);
-    C = max(C, b);
-    alive |= (b > 0 ? 1u : 0u) << l;
-  }
-  uint8_t *grow = LAYOUT == MICKEY_LAYOUT_BITSLICED_U32 ? a.out + a.offsets[g] : nullptr;
-  if (alive == 0) return;                     // every lane asks for 0 bits
-
+__device__ __forceinline__ void ragged_clock_piece(const RaggedArgs &a, const LaneTab &lt,
+                                                   uint32_t g, uint32_t *zb0, uint32_t *zb1,
+                                                   uint32_t &par, uint32_t bar, uint32_t ta,
+                                                   uint32_t tb, bool ends) {
   const size_t P = a.Gpad;
-  uint32_t *st = a.state + g;
+  const bool valid = g < a.G;
   uint32_t r[kReg], s[kReg];
+  uint32_t *st = a.state + (valid ? g : 0);
+  // lanes whose state this piece carries on: their bits leave HBM
+  const uint32_t live = valid ? lanes_where(lt.snap, [ta](uint32_t x) { return x != ~0u && x >= ta; })
+                              : 0u;
 #pragma unroll
   for (int i = 0; i < kReg; ++i) {
     r[i] = st[size_t(i) * P];
     s[i] = st[size_t(kReg + i) * P];
   }
-  // Unless every lane has the same length (one plain store of the whole group
-  // at the end), the end points OR their lanes' words in: clear those lanes.
-  if (!same_end(lt, lanes, C)) {
-#pragma unroll 1
-    for (int i = 0; i < 2 * kReg; ++i) atomicAnd(st + size_t(i) * P, ~alive);
-  }
-  uint32_t *zb0 = zs + threadIdx.x, *zb1 = zs + 32 * kRaggedThreads + threadIdx.x;
-  KgFeed fd = kg_feed<false>(r, s, 0u);
-  const uint32_t NT = uint32_t((C + 31) >> 5);      // lengths are at most 2^34
-#pragma unroll 1
-  for (uint32_t T = 0; T < NT; ++T) {
-    const uint64_t t0 = uint64_t(T) << 5;
-    uint32_t *cur = (T & 1) ? zb1 : zb0, *prev = (T & 1) ? zb0 : zb1;
-    const uint32_t ends = tile_ends(lt, lanes, t0);
-#pragma unroll 1
-    for (int c = 0; c < 32; ++c) {
-      cur[c * kRaggedThreads] = lop3<kXorAnd>(r[0], s[0], alive);  // (r0 ^ s0) & alive
-      clock_kg_from<false>(r, s, fd, 0u);
-      fd = kg_feed<false>(r, s, 0u);         // the next clock's, inside this iteration
-      if ((ends >> c) & 1u) {                  // some lanes have run their length
-        const uint32_t m = lanes_ending(lt, lanes, t0 + c + 1);
-        snapshot(st, P, r, s, m, pad);
-        alive &= ~m;
-      }
-      if ((c & 3) == 3 && T > 0)
-        ragged_slice<LAYOUT>(prev, lt, grow, lanes, t0 - 32, 32, C, c >> 2);
+  if (live) {
+    size_t Q;
+    uint32_t *wr = opaque(st, P, Q);
+#pragma unroll
+    for (int i = 0; i < kReg; ++i) {
+      wr[size_t(i) * Q] = r[i] & ~live;
+      wr[size_t(kReg + i) * Q] = s[i] & ~live;
     }
   }
-  // the last tile (possibly partial)
-  const uint64_t tl = uint64_t(NT - 1) << 5;
-  ragged_tile<LAYOUT>(((NT - 1) & 1) ? zb1 : zb0, lt, grow, lanes, tl,
-                      C - tl >= 32 ? 32 : int(C - tl), C);
+#pragma unroll 1
+  for (uint32_t T = ta;; ++T) {
+    // lanes that end before the next look; after the last tile those that end
+    // there, or, where the next segment goes on, all that run on
+    if (valid && T % kSnapTiles == 0) {      // tb too is a multiple
+      const bool hand_on = T == tb && !ends;
+      const uint32_t m = lanes_where(
+          lt.snap, [=](uint32_t x) { return x == T || (hand_on && x > T && x != ~0u); });
+      if (m) merge_lanes(st, P, r, s, m);
+    }
+    if (T == tb) break;
+    uint32_t *cur = par ? zb1 : zb0;
+#pragma unroll 1
+    for (int c = 0; c < 32; c += 4) {
+      uint32_t *row = cur + clock_row<LAYOUT>(c) * kKsThreads;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        row[u * kKsThreads] = r[0] ^ s[0];
+        clock_kg<false, false>(r, s, 0u, 0u);
+      }
+    }
+    pair_sync(bar);
+    par ^= 1u;
+  }
+}
+
+// Store the tile's words of the group's rows.  `first`: the piece's first tile;
+// `final`: the last tile of a piece that the next segment continues.  The rows
+// that go on past the tile take the loop; its code and the one copy of the
+// byte-wise cases stay small beside the clock loop in the instruction cache
+// (all 32 rows unrolled with their cases: 34.6 ms where the clocks take 10).
+template <int LAYOUT>
+__device__ __forceinline__ void ragged_rows(const RaggedArgs &a, const LaneTab &lt, uint32_t g,
+                                            uint32_t *z, uint32_t T, bool first, bool final) {
+  uint32_t m[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) m[i] = z[i * kKsThreads];
+  transpose32_prmt(m);                       // m[31 - l]: lane l's word
+#pragma unroll
+  for (int l = 0; l < 32; ++l) z[l * kKsThreads] = m[31 - l];
+  uint32_t whole = 0, ending = 0;
+#pragma unroll 4
+  for (int l = 0; l < 32; ++l) {
+    const uint32_t n_tiles = lt.tiles[l * kKsThreads];
+    ending |= (T + 1 == n_tiles ? 1u : 0u) << l;
+    if (T + 1 >= n_tiles) continue;
+    whole |= 1u << l;
+    const uint64_t base = lt.row[l * kKsThreads];
+    const uint32_t al = uint32_t(base) & 3u; // the row starts `al` bytes into its first word
+    const uint32_t w = z[l * kKsThreads], prev = lt.carry[l * kKsThreads];
+    lt.carry[l * kKsThreads] = w;
+    if (!first)
+      *reinterpret_cast<uint32_t *>(base - al + 4ull * T) = __funnelshift_l(prev, w, 8 * al);
+  }
+  // rows byte by byte: the part of the first word that is theirs, and what is
+  // left of the last one
+  for (uint32_t todo = ending | (first || final ? whole : 0u); todo; todo &= todo - 1) {
+    const int l = __ffs(int(todo)) - 1;
+    const uint64_t base = lt.row[l * kKsThreads];
+    const uint32_t al = uint32_t(base) & 3u;
+    uint8_t *o = reinterpret_cast<uint8_t *>(base - al) + 4ull * T;
+    uint32_t w = z[l * kKsThreads];
+    if ((whole >> l) & 1u) {
+      for (uint32_t b = al; first && b < 4; ++b) o[b] = uint8_t(w >> (8 * (b - al)));
+      for (uint32_t b = 0; final && b < al; ++b) o[4 + b] = uint8_t(w >> (8 * (4 - al + b)));
+    } else {
+      const int nb = int((a.n_bits[32ull * g + l] - 1) & 31u) + 1;
+      if (LAYOUT == MICKEY_LAYOUT_BYTES) w &= __byte_perm(~0u << (32 - nb), 0u, 0x0123);
+      const uint32_t prev = lt.carry[l * kKsThreads];
+      for (uint32_t b = 0; !first && b < al; ++b) o[b] = uint8_t(prev >> (8 * (4 - al + b)));
+      for (int b = 0; b < (nb + 7) >> 3; ++b) o[al + b] = uint8_t(w >> (8 * b));
+    }
+  }
+}
+
+// The tile's words of a bitsliced row (T in words of the group's longest lane).
+__device__ __forceinline__ void ragged_words(const RaggedArgs &a, const LaneTab &lt, uint32_t g,
+                                             uint32_t *z, uint32_t T, uint64_t words) {
+  uint32_t alive = 0;
+  for (int l = 0; l < 32; ++l) {
+    const uint32_t n_tiles = lt.tiles[l * kKsThreads];
+    if (T >= n_tiles) continue;
+    alive |= 1u << l;
+    if (T + 1 == n_tiles)                           // ends inside: its later clocks' bits go
+      for (int c = int((a.n_bits[32ull * g + l] - 1) & 31u) + 1; c < 32; ++c)
+        z[c * kKsThreads] &= ~(1u << l);
+  }
+  if (!alive) return;
+  uint32_t *o = reinterpret_cast<uint32_t *>(a.out + a.offsets[g]) + 32ull * T;
+  const uint64_t left = words - 32ull * T;
+  const int n = left < 32 ? int(left) : 32;
+  // vectors from the first 16-byte boundary on
+  int c = 0;
+  for (; c < n && (reinterpret_cast<uintptr_t>(o + c) & 15u); ++c) o[c] = z[c * kKsThreads] & alive;
+#pragma unroll 2
+  for (; c + 4 <= n; c += 4)
+    *reinterpret_cast<uint4 *>(o + c) =
+        make_uint4(z[c * kKsThreads] & alive, z[(c + 1) * kKsThreads] & alive,
+                   z[(c + 2) * kKsThreads] & alive, z[(c + 3) * kKsThreads] & alive);
+  for (; c < n; ++c) o[c] = z[c * kKsThreads] & alive;
+}
+
+// The warp-group that holds block x of the work line: the last w with
+// blocks[w] <= x (x below blocks[W]).
+__device__ __forceinline__ uint32_t find_group(const uint64_t *blocks, uint32_t W, uint64_t x) {
+  uint32_t lo = 0, hi = W;
+  while (hi - lo > 1) {
+    const uint32_t mid = lo + (hi - lo) / 2;
+    if (blocks[mid] <= x) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// Pieces of a segment in the order head, whole warp-groups, tail, as
+// segment_piece, on the prefix sums.  Without hand-offs (cooperative = 0)
+// slot w has warp-group w.
+__device__ __forceinline__ bool ragged_piece(const PersistArgs &p, const uint64_t *blocks,
+                                             uint32_t slot, uint32_t k, uint32_t &w, uint32_t &ta,
+                                             uint32_t &tb) {
+  if (!p.cooperative) {
+    w = slot;
+    ta = 0;
+    if (k || slot >= p.W) return false;
+    tb = kSnapTiles * uint32_t(blocks[slot + 1] - blocks[slot]);
+    return true;
+  }
+  const uint64_t total = blocks[p.W];
+  const uint64_t a = uint64_t(slot) * p.L, b = a + p.L < total ? a + p.L : total;
+  if (a >= b) return false;
+  const uint32_t wf = find_group(blocks, p.W, a), wl = find_group(blocks, p.W, b - 1);
+  const bool head = b < blocks[wl + 1] && (wl != wf || a == blocks[wf]);
+  if (head && k == 0) {
+    w = wl;
+    ta = 0;
+    tb = kSnapTiles * uint32_t(b - blocks[wl]);
+    return true;
+  }
+  k -= head ? 1 : 0;
+  const bool tail = a > blocks[wf];
+  const uint32_t lo = wf + (tail ? 1 : 0), hi = b < blocks[wl + 1] ? wl : wl + 1;   // whole: [lo, hi)
+  const uint32_t whole = hi > lo ? hi - lo : 0;
+  if (k < whole) {
+    w = lo + k;
+    ta = 0;
+    tb = kSnapTiles * uint32_t(blocks[w + 1] - blocks[w]);
+    return true;
+  }
+  if (k > whole || !tail) return false;
+  w = wf;
+  ta = kSnapTiles * uint32_t(a - blocks[wf]);
+  tb = kSnapTiles * uint32_t((b < blocks[wf + 1] ? b : blocks[wf + 1]) - blocks[wf]);
+  return true;
 }
 
 template <int LAYOUT>
-cudaError_t launch_ragged_layout(const RaggedArgs &a, cudaStream_t st) {
-  const cudaError_t e = cudaFuncSetAttribute(
-      ragged_kernel<LAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kRaggedSmem));
+__global__ void __launch_bounds__(2 * kKsThreads, 1)
+    ragged_ws_kernel(RaggedArgs a, PersistArgs p) {
+  extern __shared__ __align__(16) uint32_t zs[];
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t t = threadIdx.x & (kKsThreads - 1);
+  const uint32_t pair = t >> 5;
+  const bool clocker = threadIdx.x < kKsThreads;
+  const uint32_t slot = blockIdx.x * (kKsThreads / 32) + pair;
+  uint32_t *zb0 = zs + t, *zb1 = zs + 32 * kKsThreads + t;
+  const LaneTab lt = lane_tab(zs, t);
+  uint32_t par = 0;
+#pragma unroll 1
+  for (uint32_t k = 0;; ++k) {
+    uint32_t w, ta, tb;
+    if (!ragged_piece(p, a.blocks, slot, k, w, ta, tb)) break;
+    if (ta == tb) continue;                  // a warp-group that asks for no bits
+    const uint32_t g = w * 32 + lane;
+    const bool ends = a.blocks[w] + tb / kSnapTiles == a.blocks[w + 1];
+    if (clocker) {
+      if (ta > 0) {  // tail: wait for the head piece of this warp-group
+        uint32_t it = 0;
+        bool ok = true;
+        while (load_acquire(p.flags + w) != p.wait_epoch) {
+          if (++it > p.spin_limit) {
+            ok = false;
+            break;
+          }
+          __nanosleep(256);
+        }
+        if (!__all_sync(0xffffffffu, ok) && lane == 0) atomicOr(p.err, kErrTimeout);
+      }
+    }
+    // The lane table: the clock side fills what it reads itself (snap), the
+    // emission side the rest.  Every thread uses its own columns only.
+    uint64_t words = 0;
+    for (int l = 0; l < 32; ++l) {
+      const uint64_t i = 32ull * g + l;
+      const uint64_t n = g < a.G && i < a.n ? a.n_bits[i] : 0;
+      if (clocker) {
+        lt.snap[l * kKsThreads] = n ? uint32_t(n / kRaggedBlockBits) * kSnapTiles : ~0u;
+      } else {
+        lt.tiles[l * kKsThreads] = uint32_t((n + 31) >> 5);
+        if (LAYOUT != MICKEY_LAYOUT_BITSLICED_U32)
+          lt.row[l * kKsThreads] = n ? reinterpret_cast<uint64_t>(a.out + a.offsets[i]) : 0ull;
+        words = max(words, n);
+      }
+    }
+    if (clocker) {
+      ragged_clock_piece<LAYOUT>(a, lt, g, zb0, zb1, par, 1 + pair, ta, tb, ends);
+      if (!ends) {  // head: publish the state for the next segment
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) store_release(p.flags + w, p.epoch);
+      }
+    } else {
+#pragma unroll 1
+      for (uint32_t T = ta; T < tb; ++T) {
+        pair_sync(1 + pair);
+        uint32_t *z = par ? zb1 : zb0;
+        par ^= 1u;
+        if (32ull * T >= words) continue;    // the group's lanes have all ended
+        if constexpr (LAYOUT == MICKEY_LAYOUT_BITSLICED_U32)
+          ragged_words(a, lt, g, z, T, words);
+        else
+          ragged_rows<LAYOUT>(a, lt, g, z, T, T == ta, T == tb - 1 && !ends);
+      }
+    }
+  }
+}
+
+// The clocks that ragged_ws_kernel left: each lane's own 0 .. kRaggedBlockBits - 1,
+// a thread per instance.
+__global__ void __launch_bounds__(32) ragged_rest_kernel(RaggedArgs a) {
+  const uint32_t lane = threadIdx.x, g = blockIdx.x;
+  const uint64_t i = 32ull * g + lane;
+  const uint32_t rest = i < a.n ? uint32_t(a.n_bits[i] % kRaggedBlockBits) : 0u;
+  const uint32_t most = __reduce_max_sync(0xffffffffu, rest);
+  if (most == 0) return;
+  Packed q;
+  packed_load(q, a.state, a.Gpad, g, lane);
+#pragma unroll 1
+  for (uint32_t c = 0; c < most; c += 8) {
+    if (__all_sync(0xffffffffu, c + 8 <= rest)) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) clock_packed<false>(q, 0u);
+    } else {
+#pragma unroll 1
+      for (uint32_t u = c; u < c + 8; ++u)
+        if (u < rest) clock_packed<false>(q, 0u);
+    }
+  }
+  packed_store(q, a.state, a.Gpad, g, lane);
+}
+
+// ---------------------------------------------------- one thread per instance
+
+template <int LAYOUT>
+__global__ void __launch_bounds__(32) ragged_packed_kernel(RaggedArgs a) {
+  const uint32_t lane = threadIdx.x, g = blockIdx.x;
+  const uint64_t i = 32ull * g + lane;
+  const uint64_t n = i < a.n ? a.n_bits[i] : 0;
+  if (__all_sync(0xffffffffu, n == 0)) return;
+  const uint64_t full = n >> 5;
+  const int rem = int(n & 31);
+  Packed q;
+  packed_load(q, a.state, a.Gpad, g, lane);
+  if constexpr (LAYOUT == MICKEY_LAYOUT_BITSLICED_U32) {
+    uint32_t *o = reinterpret_cast<uint32_t *>(a.out + a.offsets[g]);
+    const uint32_t tiles = __reduce_max_sync(0xffffffffu, uint32_t((n + 31) >> 5));
+    const uint32_t ends = __reduce_max_sync(0xffffffffu, (n + 31) >> 5 == tiles ? uint32_t((n - 1) & 31) + 1 : 0u);
+#pragma unroll 1
+    for (uint32_t t = 0; t < tiles; ++t) {
+      uint32_t z = 0;
+      if (t < full) z = packed_clocks<32>(q);
+      else if (t == full && rem) z = packed_tail(q, rem);
+      __syncwarp();
+      z = warp_transpose(__brev(z), lane);
+      if (t + 1 < tiles || lane < ends) o[32ull * t + lane] = z;
+    }
+  } else {
+    RowOut row(n ? a.out + a.offsets[i] : nullptr, false, n != 0);
+#pragma unroll 1
+    for (uint64_t t = 0; t < full; ++t) {
+      const uint32_t z = packed_clocks<32>(q);
+      row.put(t, LAYOUT == MICKEY_LAYOUT_BYTES ? __byte_perm(z, 0u, 0x0123) : z);
+    }
+    const uint32_t z = rem ? packed_tail(q, rem) : 0u;
+    row.finish(full, (rem + 7) >> 3, __byte_perm(z, 0u, 0x0123));
+    __syncwarp();
+  }
+  packed_store(q, a.state, a.Gpad, g, lane);
+}
+
+template <int LAYOUT>
+cudaError_t launch_layout(const RaggedArgs &a, const PersistArgs *p, cudaStream_t st) {
+  if (!p) {
+    ragged_packed_kernel<LAYOUT><<<a.G, 32, 0, st>>>(a);
+    return cudaGetLastError();
+  }
+  cudaError_t e = cudaFuncSetAttribute(
+      ragged_ws_kernel<LAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kRaggedSmem));
   if (e != cudaSuccess) return e;
-  const uint32_t blocks = (a.G + kRaggedThreads - 1) / kRaggedThreads;
-  ragged_kernel<LAYOUT><<<blocks, kRaggedThreads, kRaggedSmem, st>>>(a);
+  cudaLaunchConfig_t cfg = {};
+  cfg.dynamicSmemBytes = kRaggedSmem;
+  cfg.gridDim = dim3(p->blocks);
+  cfg.blockDim = dim3(2 * kKsThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = p->cooperative ? 1 : 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, ragged_ws_kernel<LAYOUT>, a, *p);
+  if (e != cudaSuccess) return e;
+  ragged_rest_kernel<<<a.G, 32, 0, st>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_ragged(const RaggedArgs &a, int layout, cudaStream_t st) {
+cudaError_t launch_ragged(const RaggedArgs &a, int layout, const PersistArgs *p, cudaStream_t st) {
   switch (layout) {
-    case MICKEY_LAYOUT_BITSLICED_U32: return launch_ragged_layout<MICKEY_LAYOUT_BITSLICED_U32>(a, st);
-    case MICKEY_LAYOUT_BYTES: return launch_ragged_layout<MICKEY_LAYOUT_BYTES>(a, st);
-    case MICKEY_LAYOUT_U32: return launch_ragged_layout<MICKEY_LAYOUT_U32>(a, st);
+    case MICKEY_LAYOUT_BITSLICED_U32: return launch_layout<MICKEY_LAYOUT_BITSLICED_U32>(a, p, st);
+    case MICKEY_LAYOUT_BYTES: return launch_layout<MICKEY_LAYOUT_BYTES>(a, p, st);
+    case MICKEY_LAYOUT_U32: return launch_layout<MICKEY_LAYOUT_U32>(a, p, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -234,3 +234,55 @@ def test_bitsliced_rows_off_the_16_byte_grid(monkeypatch, n_bits):
     want = oracle.batch_bytes(s.keys, s.ivs, s.iv_lens, n_bits, threads=THREADS)
     got = _streams(s).generate(n_bits, "bitsliced").cpu().numpy().view(np.uint32)
     assert np.array_equal(got, oracle.to_bitsliced(want, n_bits))
+
+
+def _ragged_lengths(n, layout, seed):
+    rng = np.random.default_rng(seed)
+    nb = rng.integers(0, 700, n).astype(np.uint64)
+    nb[:24] = [0, 1, 7, 31, 32, 33, 64, 95, 96, 97, 127, 128, 129, 159, 160, 161, 255, 256, 257, 384,
+               512, 639, 640, 641]
+    nb[1024:2048] = rng.integers(0, 40, 1024)      # a warp-group of short lanes
+    if n > 3072:
+        nb[2048:3072] = 0                          # one that asks for nothing
+    return nb // 32 * 32 if layout == "u32" else nb
+
+
+# 3 warp-groups on pairs of their own; 6 on 4 clock warps, which hand states on
+@pytest.mark.parametrize("n", [2 * 1024 + 70, 6 * 1024 - 9])
+@pytest.mark.parametrize("layout", ["bytes", "u32", "bitsliced"])
+def test_ragged_thread_per_group_and_per_instance_agree(monkeypatch, n, layout):
+    s = _mixed(n)
+    handles = [_streams(s)]                        # few groups: a thread per instance
+    monkeypatch.setenv("MICKEY_MODE", "persistent")
+    monkeypatch.setenv("MICKEY_PERSIST_BLOCKS", "1")
+    handles.append(_streams(s))                    # a thread per group
+    for call in range(3):
+        nb = _ragged_lengths(n, layout, 10 * n + call)
+        if layout == "bytes" and call == 2:        # rows at any byte, gaps between them
+            gaps = np.random.default_rng(1).integers(0, 6, n).astype(np.uint64)
+            offs = np.cumsum((nb + np.uint64(7)) // np.uint64(8) + gaps) - (
+                (nb + np.uint64(7)) // np.uint64(8))
+            size = int(offs[-1]) + 200
+        else:
+            offs, size = None, int(nb.sum()) // 8 + n + 64
+            if layout == "bitsliced":
+                size = 4 * 700 * ((n + 31) // 32)
+        outs = []
+        for h in handles:
+            out = torch.full((size,), 0x5A, dtype=torch.uint8, device="cuda")
+            h.generate_ragged(nb, layout, out=out, offsets=offs)
+            h.sync()
+            outs.append(out)
+        assert torch.equal(*outs)
+    states, positions = zip(*(h.export_state() for h in handles))
+    assert np.array_equal(*states) and np.array_equal(*positions)
+    # and the oracle, over the state both ended in: the next bits of some streams
+    idx = np.arange(0, n, 37)
+    nxt = [h.generate(64, "bytes").cpu().numpy()[idx] for h in handles]
+    want = oracle.batch_bytes(s.keys[idx], s.ivs[idx], s.iv_lens[idx],
+                              positions[0][idx] + np.uint64(64), threads=THREADS)
+    for k, i in enumerate(idx):
+        lo = int(positions[0][i])
+        bits = np.unpackbits(np.asarray(want[k]))[lo:lo + 64]
+        assert np.array_equal(np.packbits(bits), nxt[0][k])
+        assert np.array_equal(nxt[0][k], nxt[1][k])
