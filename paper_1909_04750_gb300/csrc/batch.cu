@@ -179,35 +179,30 @@ __device__ __forceinline__ void store_row(uint8_t *o, uint64_t bits, uint32_t t,
 }
 
 // One warp per group (split path), a stream per lane (packed.cuh): the group
-// runs as long as its longest lane.  Rows that start 16-byte aligned are
-// written four tiles at a time while the lane has them whole.  Not inlined:
-// as a function of its own it gets a register allocation of its own instead
-// of sharing the one-thread-per-group path's 255.
-__device__ __noinline__ void packed_group(const uint32_t *state, size_t P, uint32_t g,
-                                          uint64_t clocks, uint8_t *row, uint64_t bits,
-                                          uint32_t lane) {
+// runs as long as its longest lane.
+__device__ __forceinline__ void packed_group(const uint32_t *state, size_t P, uint32_t g,
+                                             uint64_t clocks, uint8_t *row, uint64_t bits,
+                                             uint32_t lane) {
   Packed q;
   packed_load(q, state, P, g, lane);
-  const uint32_t full = uint32_t(clocks >> 5);
-  const bool vec = (reinterpret_cast<uintptr_t>(row) & 15u) == 0;
-  uint4 v = make_uint4(0u, 0u, 0u, 0u);
+  const uint32_t full = uint32_t(clocks >> 5), whole = uint32_t(bits >> 5);
+  uint32_t *o = reinterpret_cast<uint32_t *>(row);
 #pragma unroll 1
   for (uint32_t t = 0; t < full; ++t) {
     const uint32_t w = __byte_perm(packed_clocks<32>(q), 0u, 0x0123);
-    v = make_uint4(v.y, v.z, v.w, w);
-    if (!vec) {
-      store_row(row, bits, t, w);
-    } else if ((t & 3) == 3 && (uint64_t(t) + 1) * 32 <= bits) {
-      *reinterpret_cast<uint4 *>(row + 4ull * (t - 3)) = v;
-    } else if ((t & 3) == 3 || t == full - 1) {   // a block of four that ends early
-      const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (uint32_t j = 0; j < 4; ++j)
-        if (3 - j <= (t & 3)) store_row(row, bits, t - (3 - j), w4[j]);
-    }
+    if (t < whole) o[t] = w;
+    else store_row(row, bits, t, w);       // the lane ends in this tile, or has
   }
   const int rem = int(clocks & 31);
   if (rem) store_row(row, bits, full, __byte_perm(packed_tail(q, rem), 0u, 0x0123));
+}
+
+// In the persistent kernel as a function of its own, with a register
+// allocation of its own instead of the one-thread-per-group path's 255.
+__device__ __noinline__ void packed_group_call(const uint32_t *state, size_t P, uint32_t g,
+                                               uint64_t clocks, uint8_t *row, uint64_t bits,
+                                               uint32_t lane) {
+  packed_group(state, P, g, clocks, row, bits, lane);
 }
 
 // Split kernel: one-warp blocks take the split groups (0 .. n_split-1,
@@ -243,7 +238,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(BatchArgs a) {
     if (item >= a.n_items) break;
     if (item < a.split_items) {
       const uint64_t slot = uint64_t(item) * 32 + lane;
-      packed_group(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
+      packed_group_call(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
                    a.slot_bits[slot], lane);
       continue;
     }
@@ -301,7 +296,7 @@ void batch_release(mickey_batch *b) {
 
 // Time per clock (ns) of a split warp when 1, 2, 3 or 4 share an SM
 // sub-partition (row stores included).
-constexpr double kPackedNs[4] = {32.0, 55.0, 78.0, 102.0};
+constexpr double kPackedNs[4] = {29.0, 52.0, 76.0, 100.0};
 // Up to this many groups per SM a new plan splits every group.  A thread item
 // clocks 32 groups at 820 ns per clock (1140 when two share a sub-partition),
 // so it wins only once there are items for every warp and their lengths are

@@ -34,11 +34,12 @@ __device__ __forceinline__ void packed_store_word(uint8_t *o, uint64_t f32_off, 
 }
 
 // Keystream of group blockIdx.x, one instance per lane.  The row layouts
-// store four tiles of a row at once (16 bytes) where rows and output are
-// 16-byte aligned, else a word or bytes per tile; the bitsliced layout turns
-// each tile round with a transpose across the warp.
+// store a word (or bytes, off the word grid) per tile; the bitsliced layout
+// turns each tile round with a transpose across the warp.  The loop around
+// packed_clocks holds nothing else: with four tiles' words kept for 16-byte
+// stores the compiler's schedule of the clocks was 16 % slower.
 template <int LAYOUT>
-__global__ void __launch_bounds__(kPackedThreads)
+__global__ void __launch_bounds__(32)
     packed_keystream_kernel(KeystreamArgs a, uint32_t lane_mask) {
   const uint32_t lane = threadIdx.x, g = blockIdx.x;
   if (g != a.G - 1) lane_mask = ~0u;
@@ -62,23 +63,10 @@ __global__ void __launch_bounds__(kPackedThreads)
     const uint64_t pitch = LAYOUT == MICKEY_LAYOUT_BYTES ? (a.n_bits + 7) >> 3 : a.n_bits >> 3;
     const uint64_t f32_off = pitch * a.n;
     uint8_t *o = static_cast<uint8_t *>(a.out) + (32ull * g + lane) * pitch;
-    const bool vec = (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0 && a.n_bits % 128 == 0;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
     for (uint64_t t = 0; t < full; ++t) {
       const uint32_t z = packed_clocks<32>(q);
-      if (!vec) {
-        if (valid) packed_store_word<LAYOUT>(o, f32_off, t, 32, z);
-        continue;
-      }
-      v = make_uint4(v.y, v.z, v.w, LAYOUT == MICKEY_LAYOUT_BYTES ? __byte_perm(z, 0u, 0x0123) : z);
-      if ((t & 3) == 3 && valid) {   // vec: full is a multiple of 4
-        *reinterpret_cast<uint4 *>(o + 4 * (t - 3)) = v;
-        if constexpr (LAYOUT == MICKEY_LAYOUT_U32_F32)
-          *reinterpret_cast<float4 *>(o + f32_off + 4 * (t - 3)) = make_float4(
-              __uint2float_rn(v.x >> 8) * 0x1p-24f, __uint2float_rn(v.y >> 8) * 0x1p-24f,
-              __uint2float_rn(v.z >> 8) * 0x1p-24f, __uint2float_rn(v.w >> 8) * 0x1p-24f);
-      }
+      if (valid) packed_store_word<LAYOUT>(o, f32_off, t, 32, z);
     }
     if (rem) {
       const uint32_t z = packed_tail(q, rem);

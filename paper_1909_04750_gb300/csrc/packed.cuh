@@ -22,12 +22,15 @@
 // words k2 + fb (FB0 part) + fb cbs (FB1 part) (each bit a 0/1 times a
 // constant, differences mod 2^32), fb_R x RTAPS and cb_R x r_i.  That leaves
 // 22 logic and 23 multiply-add operations per clock of 32 instances.
-// Measured (GB300, 2.07 GHz, clocks alone): 29.4 ns per clock for a lone
-// warp, 31.3 with one warp per SM sub-partition, 782 Gbit/s with eight;
-// with the R update in logic operations 29.8 / 31.1 ns and 717 Gbit/s.  The
-// column form spread over a warp's lanes (four bits of each register per
-// lane, seven shuffles per clock), which this one replaces, took 34.2 ns and
-// at most 649 Gbit/s; one thread per 32-lane group takes 334 ns.
+// Measured (GB300, 2.07 GHz, with the row stores): 26.0 ns per clock for a lone
+// warp, 27.6 with one warp per SM sub-partition; clocks alone 782 Gbit/s with
+// eight (717 with the R update in logic operations).  The logic pipe would
+// allow 21.3 ns; the rest is the schedule, which the compiler does best in a
+// one-warp kernel whose loop holds the 32 clocks and a word store (control
+// bits' words written first; other orders, register bounds or four words kept
+// for a vector store: 28 to 44 ns).  The column form spread over a warp's
+// lanes, which this one replaces, took 34.2 ns and at most 649 Gbit/s; one
+// thread per 32-lane group takes 334 ns.
 #pragma once
 
 #include <cstdint>
@@ -72,43 +75,63 @@ constexpr PackedMasks make_packed_masks() {
 }
 constexpr PackedMasks kPackedMasks = make_packed_masks();
 
-// One CLOCK_KG of the thread's instance; MIX as in clock_kg, `in` 0 or 1.
+// The control and feedback bits of a clock: CONTROL_BIT_R (0 / 1), FB_R (0 /
+// ~0), FB_S and FB_S & CONTROL_BIT_S (0 / 1).
+struct PackedCtl {
+  uint32_t cbr, fbr, fbs, fc;
+};
+
+// MIX as in clock_kg, `in` 0 or 1.
+template <bool MIX>
+__device__ __forceinline__ PackedCtl packed_ctl(const Packed &q, uint32_t in) {
+  static_assert(!packed_c0(34) && packed_c0(67) && !packed_c0(50), "control bits as held");
+  PackedCtl c;
+  c.fbs = MIX ? (q.a[0] ^ in) & 1u : q.a[0] & 1u;
+  const uint32_t ncbs = (q.a[0] ^ q.r[1]) >> 8;            // bit 0: NOT CONTROL_BIT_S
+  c.fc = lop3<0x20>(c.fbs, ncbs, 1u);                      // fbs & ~ncbs & 1
+  c.cbr = ((q.a[1] ^ q.r[3]) >> 16) & 1u;
+  c.fbr = MIX ? 0u - (((q.r[3] >> 24) ^ (q.a[1] >> 12) ^ in) & 1u)   // r99 ^ s50 ^ in
+              : uint32_t(int32_t(q.r[3] << 7) >> 31);
+  return c;
+}
+
+template <int W>
+__device__ __forceinline__ uint32_t packed_r(const Packed &q, const PackedCtl &c) {
+  constexpr uint32_t tap = 0u - kPackedMasks.tap[W];
+  const uint32_t rm1 = W ? q.r[(W + 3) % 4] : q.r[3] << 1;                 // r_{i-1}
+  return lop3<0x96>(rm1, mad32(q.r[W], c.cbr, 0u), mad32(c.fbr, tap, 0u));
+}
+template <int W>
+__device__ __forceinline__ uint32_t packed_a(const Packed &q, const PackedCtl &c) {
+  constexpr uint32_t k = kPackedMasks.k[W], k2 = kPackedMasks.k2[W], x = kPackedMasks.x[W],
+                     y = kPackedMasks.y[W];
+  const uint32_t sp1 = W ? q.a[(W + 3) % 4] : q.a[3] << 1;                 // a_{i+1}
+  const uint32_t sm1 = W < 2    ? q.a[(W + 1) % 4]                         // a_{i-1}
+                       : W == 2 ? mad32(q.s0, 1u << 24, q.a[3])
+                                : q.a[0] >> 1;
+  return lop3<0x96>(lop3<0x60>(q.a[W], sp1, k), sm1, mad32(c.fc, y, mad32(c.fbs, x, k2)));
+}
+
+// The registers one clock on.  The words that the next clock's control bits
+// come from are written first.
+__device__ __forceinline__ Packed packed_step(const Packed &q, const PackedCtl &c) {
+  Packed n;
+  n.a[0] = packed_a<0>(q, c);
+  n.a[1] = packed_a<1>(q, c);
+  n.r[1] = packed_r<1>(q, c);
+  n.r[3] = packed_r<3>(q, c);
+  n.a[2] = packed_a<2>(q, c);
+  n.r[0] = packed_r<0>(q, c);
+  n.s0 = c.fbs;
+  n.a[3] = packed_a<3>(q, c);
+  n.r[2] = packed_r<2>(q, c);
+  return n;
+}
+
+// One CLOCK_KG of the thread's instance.
 template <bool MIX>
 __device__ __forceinline__ void clock_packed(Packed &q, uint32_t in) {
-  static_assert(!packed_c0(34) && packed_c0(67) && !packed_c0(50), "control bits as held");
-  uint32_t(&r)[4] = q.r;
-  uint32_t(&a)[4] = q.a;
-  const uint32_t cbr = ((a[1] ^ r[3]) >> 16) & 1u;   // CONTROL_BIT_R
-  uint32_t fbr, fbs;                                 // fbr: 0 or ~0; fbs: 0 or 1
-  if constexpr (MIX) {
-    fbr = 0u - (((r[3] >> 24) ^ (a[1] >> 12) ^ in) & 1u);   // r99 ^ s50 ^ in
-    fbs = (a[0] ^ in) & 1u;
-  } else {
-    fbr = uint32_t(int32_t(r[3] << 7) >> 31);
-    fbs = a[0] & 1u;
-  }
-  const uint32_t ncbs = (a[0] ^ r[1]) >> 8;          // bit 0: NOT CONTROL_BIT_S
-  const uint32_t fc = lop3<0x20>(fbs, ncbs, 1u);     // fbs & ~ncbs & 1
-  uint32_t nr[4], na[4];
-  static_for<0, 4>([&](auto wc) {
-    constexpr int w = decltype(wc)::value;
-    constexpr uint32_t tap = 0u - kPackedMasks.tap[w], k = kPackedMasks.k[w],
-                       k2 = kPackedMasks.k2[w], x = kPackedMasks.x[w], y = kPackedMasks.y[w];
-    const uint32_t rm1 = w ? r[(w + 3) % 4] : r[3] << 1;                  // r_{i-1}
-    nr[w] = lop3<0x96>(rm1, mad32(r[w], cbr, 0u), mad32(fbr, tap, 0u));
-    const uint32_t sp1 = w ? a[(w + 3) % 4] : a[3] << 1;                  // a_{i+1}
-    const uint32_t sm1 = w < 2    ? a[(w + 1) % 4]                        // a_{i-1}
-                         : w == 2 ? mad32(q.s0, 1u << 24, a[3])
-                                  : a[0] >> 1;
-    const uint32_t v = lop3<0x60>(a[w], sp1, k);                          // a & (sp1 ^ k)
-    na[w] = lop3<0x96>(v, sm1, mad32(fc, y, mad32(fbs, x, k2)));
-  });
-#pragma unroll
-  for (int w = 0; w < 4; ++w) {
-    r[w] = nr[w];
-    a[w] = na[w];
-  }
-  q.s0 = fbs;
+  q = packed_step(q, packed_ctl<MIX>(q, in));
 }
 
 // The zero state.

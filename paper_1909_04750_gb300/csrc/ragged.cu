@@ -394,14 +394,22 @@ __global__ void __launch_bounds__(32) ragged_packed_kernel(RaggedArgs a) {
       if (t + 1 < tiles || lane < ends) o[32ull * t + lane] = z;
     }
   } else {
-    RowOut row(n ? a.out + a.offsets[i] : nullptr, false, n != 0);
+    uint8_t *o = n ? a.out + a.offsets[i] : nullptr;
+    const bool words = (reinterpret_cast<uintptr_t>(o) & 3u) == 0;
 #pragma unroll 1
-    for (uint64_t t = 0; t < full; ++t) {
+    for (uint64_t t = 0; t < full; ++t, o += 4) {
       const uint32_t z = packed_clocks<32>(q);
-      row.put(t, LAYOUT == MICKEY_LAYOUT_BYTES ? __byte_perm(z, 0u, 0x0123) : z);
+      const uint32_t w = LAYOUT == MICKEY_LAYOUT_BYTES ? __byte_perm(z, 0u, 0x0123) : z;
+      if (words) {
+        *reinterpret_cast<uint32_t *>(o) = w;
+      } else {
+        for (int b = 0; b < 4; ++b) o[b] = uint8_t(w >> (8 * b));
+      }
     }
-    const uint32_t z = rem ? packed_tail(q, rem) : 0u;
-    row.finish(full, (rem + 7) >> 3, __byte_perm(z, 0u, 0x0123));
+    if (rem) {
+      const uint32_t w = __byte_perm(packed_tail(q, rem), 0u, 0x0123);
+      for (int b = 0; b < (rem + 7) >> 3; ++b) o[b] = uint8_t(w >> (8 * b));
+    }
     __syncwarp();
   }
   packed_store(q, a.state, a.Gpad, g, lane);
