@@ -179,18 +179,6 @@ __global__ void __launch_bounds__(TB)
   }
 }
 
-// CRC-8 of 32 messages per thread (group g = messages 32g .. 32g+31),
-// general form (any length and alignment): per pass the thread loads 16
-// bytes of each of its 32 messages into registers, transposes each 32 x 32
-// bit block (one word per message -> one word per message bit, lane l =
-// message l) and clocks the bitsliced register once per bit, bytes in
-// order and each byte's most significant bit first.  Each pass uses half of
-// a 32-byte sector and leaves the other half to the next pass, which at
-// full size mostly finds it evicted from L2: the aligned form below is the
-// fast path.
-constexpr int kCrcThreads = 64;
-constexpr int kCrcChunk = 16;
-
 // Message m0 + l's CRC: bit k from s[k], lane l; then the final XOR.
 __device__ __forceinline__ void store_crcs(const uint32_t (&s)[8], size_t m0, size_t n,
                                            uint32_t xorout, uint8_t *crc) {
@@ -204,65 +192,7 @@ __device__ __forceinline__ void store_crcs(const uint32_t (&s)[8], size_t m0, si
   }
 }
 
-__device__ __forceinline__ uint4 load_chunk(const uint8_t *src, size_t left, bool vec) {
-  if (vec && left >= 16) return *reinterpret_cast<const uint4 *>(src);
-  uint32_t w[4] = {0u, 0u, 0u, 0u};
-  for (int k = 0; k < 16; ++k)
-    if (size_t(k) < left) w[k >> 2] |= uint32_t(src[k]) << (8 * (k & 3));
-  return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-__global__ void __launch_bounds__(kCrcThreads)
-    crc8_regs_kernel(const uint8_t *data, size_t n, size_t len, uint32_t poly, uint32_t init,
-                     uint32_t xorout, uint8_t *crc, bool vec, size_t G) {
-  uint32_t pm[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) pm[k] = (poly >> k) & 1u ? ~0u : 0u;
-#pragma unroll 1
-  for (size_t g = blockIdx.x * size_t(kCrcThreads) + threadIdx.x; g < G;
-       g += size_t(gridDim.x) * kCrcThreads) {
-    const size_t m0 = g * 32;
-    uint32_t s[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s[k] = (init >> k) & 1u ? ~0u : 0u;
-#pragma unroll 1
-    for (size_t off = 0; off < len; off += kCrcChunk) {
-      const size_t left = len - off;
-      uint4 v[32];
-#pragma unroll
-      for (int l = 0; l < 32; ++l)
-        v[l] = m0 + l < n ? load_chunk(data + (m0 + l) * len + off, left, vec)
-                          : make_uint4(0u, 0u, 0u, 0u);
-      const int cb = left < size_t(kCrcChunk) ? int(left) : kCrcChunk;   // uniform
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        if (4 * w < cb) {
-          uint32_t a[32];
-#pragma unroll
-          for (int l = 0; l < 32; ++l)
-            a[31 - l] = w == 0 ? v[l].x : w == 1 ? v[l].y : w == 2 ? v[l].z : v[l].w;
-          transpose32_prmt(a);   // a[c]: bit 31 - c of the word, lane l = message l
-          const int nbytes = cb - 4 * w < 4 ? cb - 4 * w : 4;
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            if (b < nbytes) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {   // byte b, most significant bit first
-                const uint32_t f = s[7] ^ a[24 - 8 * b + i];
-#pragma unroll
-                for (int k = 7; k > 0; --k) s[k] = lop3<0x78>(s[k - 1], f, pm[k]);
-                s[0] = f & pm[0];
-              }
-            }
-          }
-        }
-      }
-    }
-    store_crcs(s, m0, n, xorout, crc);
-  }
-}
-
-// Aligned form (16-byte aligned messages, len % 16 == 0): a block of
+// CRC-8 of many short aligned messages (16-byte aligned, len % 16 == 0): a block of
 // kCrcGroups threads owns kCrcGroups * 32 messages; per pass cp.async copies
 // 32 bytes (one whole sector) of each straight into shared memory, about 64
 // asynchronous 16-byte copies per thread in flight and no registers held.
@@ -446,31 +376,77 @@ __device__ __forceinline__ void crc_byte(uint32_t (&c)[8], const uint32_t (&m)[8
   for (int j = 0; j < 8; ++j) c[j] = y[j];
 }
 
-template <uint32_t POLY>
+// ANY: any length and alignment.  The warp reads the message's whole 16-byte
+// aligned units, the last of them in lane 31 of the last chunk (units that a
+// message does not have count as zeros, which change nothing in front of it);
+// lane l takes message l's bytes before its first unit and behind its last
+// one, a table step per byte (256 bytes of shared memory).  The register after
+// the front bytes goes past the units as r x^(128 U) mod P, U one of two
+// values (CrcPast).  No load is shifted or split, whatever the alignment.
+struct CrcPast {
+  uint32_t k[2];   // x^(128 U) mod P for U = len / 16 and one less
+};
+
+// table[i] = i x^8 mod P, by the whole block.
+__device__ __forceinline__ void crc_table(uint8_t *table, uint32_t poly) {
+  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) {
+    uint32_t r = i;
+#pragma unroll 1
+    for (int b = 0; b < 8; ++b) r = (r << 1) ^ ((r >> 7) & 1u ? 0x100u | poly : 0u);
+    table[i] = uint8_t(r);
+  }
+  __syncthreads();
+}
+
+// Register r past the bytes [p, end).
+__device__ __forceinline__ uint32_t crc_bytes(const uint8_t *table, uint32_t r, const uint8_t *p,
+                                              const uint8_t *end) {
+#pragma unroll 1
+  for (; p < end; ++p) r = table[r ^ *p];
+  return r;
+}
+
+template <uint32_t POLY, bool ANY>
 __global__ void __launch_bounds__(kCrcWarpBlock)
     crc8_warp_kernel(const uint8_t *data, size_t n, size_t len, uint32_t poly, uint32_t init,
-                     uint32_t xorout, uint8_t *crc, CrcJoin cj, size_t G) {
+                     uint32_t xorout, uint8_t *crc, CrcJoin cj, CrcPast past, size_t G) {
   constexpr uint32_t F = 0xffffffffu;
   const uint32_t lane = threadIdx.x & 31u;
   uint32_t pm[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) pm[k] = (poly >> k) & 1u ? ~0u : 0u;
   const size_t warps = size_t(gridDim.x) * (kCrcWarpBlock / 32);
+  const size_t span = ANY ? (len / 16 + 31) / 32 * 512 : len;
+  __shared__ uint8_t table[ANY ? 256 : 1];
+  if constexpr (ANY) crc_table(table, poly);
 #pragma unroll 1
   for (size_t g = size_t(blockIdx.x) * (kCrcWarpBlock / 32) + (threadIdx.x >> 5); g < G;
        g += warps) {
     const size_t m0 = g * 32;
     uint32_t acc[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = lane == 31 && ((init >> k) & 1u) ? ~0u : 0u;
+    for (int k = 0; k < 8; ++k) acc[k] = !ANY && lane == 31 && ((init >> k) & 1u) ? ~0u : 0u;
 #pragma unroll 1
-    for (size_t off = 0; off < len; off += 512) {
+    for (size_t off = 0; off < span; off += 512) {
       uint4 v[32];
+      if constexpr (ANY) {
+        // this lane's unit of message l lies 16 (lane's units after it) before
+        // the message's last one
+        const size_t after = span - off - 16 * lane;
+        uintptr_t first = reinterpret_cast<uintptr_t>(data) + m0 * len;   // of message l
 #pragma unroll
-      for (int l = 0; l < 32; ++l)
-        v[l] = m0 + l < n
-                   ? *reinterpret_cast<const uint4 *>(data + (m0 + l) * len + off + 16 * lane)
-                   : make_uint4(0u, 0u, 0u, 0u);
+        for (int l = 0; l < 32; ++l, first += len) {
+          const uintptr_t u = ((first + len) & ~uintptr_t(15)) - after;
+          v[l] = m0 + l < n && u >= first ? *reinterpret_cast<const uint4 *>(u)
+                                          : make_uint4(0u, 0u, 0u, 0u);
+        }
+      } else {
+#pragma unroll
+        for (int l = 0; l < 32; ++l)
+          v[l] = m0 + l < n
+                     ? *reinterpret_cast<const uint4 *>(data + (m0 + l) * len + off + 16 * lane)
+                     : make_uint4(0u, 0u, 0u, 0u);
+      }
       uint32_t c[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
@@ -514,18 +490,72 @@ __global__ void __launch_bounds__(kCrcWarpBlock)
     uint32_t r = 0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) r |= ((__shfl_sync(F, acc[k], 0) >> lane) & 1u) << k;
+    if constexpr (ANY) {
+      if (m0 + lane < n) {
+        const uint8_t *first = data + (m0 + lane) * len, *end = first + len;
+        const uint8_t *u0 = reinterpret_cast<const uint8_t *>(
+            (reinterpret_cast<uintptr_t>(first) + 15) & ~uintptr_t(15));
+        const uint8_t *u1 =
+            reinterpret_cast<const uint8_t *>(reinterpret_cast<uintptr_t>(end) & ~uintptr_t(15));
+        const bool units = u1 > u0;
+        uint32_t c = crc_bytes(table, init, first, units ? u0 : end);
+        if (units) {
+          const uint32_t k = past.k[size_t(u1 - u0) == (len & ~size_t(15)) ? 0 : 1];
+          uint32_t y = 0;                             // c k mod P
+#pragma unroll
+          for (int b = 7; b >= 0; --b) {
+            y = (y << 1) ^ ((y >> 7) & 1u ? 0x100u | poly : 0u);
+            y ^= (k >> b) & 1u ? c : 0u;
+          }
+          r = crc_bytes(table, r ^ y, u1, end);
+        } else {
+          r = c;
+        }
+      }
+    }
     if (m0 + lane < n) crc[m0 + lane] = uint8_t(r ^ xorout);
+  }
+}
+
+// Short messages of any length and alignment: a thread per message, a table
+// step per byte.
+constexpr int kCrcTableThreads = 256;
+__global__ void __launch_bounds__(kCrcTableThreads)
+    crc8_table_kernel(const uint8_t *data, size_t n, size_t len, uint32_t poly, uint32_t init,
+                      uint32_t xorout, uint8_t *crc) {
+  __shared__ uint8_t table[256];
+  crc_table(table, poly);
+  for (size_t m = size_t(blockIdx.x) * kCrcTableThreads + threadIdx.x; m < n;
+       m += size_t(gridDim.x) * kCrcTableThreads) {
+    const uint8_t *p = data + m * len;
+    crc[m] = uint8_t(crc_bytes(table, init, p, p + len) ^ xorout);
   }
 }
 
 // Polynomials with a compile-time kernel (the CRC-8 variants in common use);
 // any other runs the run-time-mask kernel.
 template <uint32_t POLY>
-void launch_crc_warp(uint32_t grid, cudaStream_t st, const uint8_t *d, size_t n, size_t len,
-                     uint32_t poly, uint32_t init, uint32_t xorout, uint8_t *crc,
-                     const CrcJoin &cj, size_t G) {
-  crc8_warp_kernel<POLY><<<grid, kCrcWarpBlock, 0, st>>>(d, n, len, poly, init, xorout, crc, cj,
-                                                         G);
+void launch_crc_warp_poly(bool any, uint32_t grid, cudaStream_t st, const uint8_t *d, size_t n,
+                          size_t len, uint32_t poly, uint32_t init, uint32_t xorout, uint8_t *crc,
+                          const CrcJoin &cj, const CrcPast &past, size_t G) {
+  if (any)
+    crc8_warp_kernel<POLY, true><<<grid, kCrcWarpBlock, 0, st>>>(d, n, len, poly, init, xorout,
+                                                                 crc, cj, past, G);
+  else
+    crc8_warp_kernel<POLY, false><<<grid, kCrcWarpBlock, 0, st>>>(d, n, len, poly, init, xorout,
+                                                                  crc, cj, past, G);
+}
+template <class... A>
+void launch_crc_warp(uint8_t poly, A &&...a) {
+  switch (poly) {
+    case 0x07: return launch_crc_warp_poly<0x07>(a...);
+    case 0x1D: return launch_crc_warp_poly<0x1D>(a...);
+    case 0x2F: return launch_crc_warp_poly<0x2F>(a...);
+    case 0x31: return launch_crc_warp_poly<0x31>(a...);
+    case 0x9B: return launch_crc_warp_poly<0x9B>(a...);
+    case 0xD5: return launch_crc_warp_poly<0xD5>(a...);
+    default: return launch_crc_warp_poly<0>(a...);
+  }
 }
 
 // Host: x^e mod P over GF(2) (P with its x^8 term), bit k = coefficient of x^k.
@@ -548,6 +578,12 @@ uint32_t gf2_xpow(uint64_t e, uint32_t P) {
     e >>= 1;
   }
   return r;
+}
+
+CrcPast crc_past(uint8_t poly, size_t len) {
+  const uint32_t P = 0x100u | poly;
+  const uint64_t U = len / 16;
+  return CrcPast{{gf2_xpow(128 * U, P), U ? gf2_xpow(128 * (U - 1), P) : 1u}};
 }
 
 CrcJoin crc_join_matrices(uint8_t poly) {
@@ -670,23 +706,28 @@ MICKEY_API int mickey_crc8(const uint8_t *data, size_t n, size_t len, uint8_t po
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const bool vec = len % 16 == 0 && reinterpret_cast<uintptr_t>(d_data) % 16 == 0;
-  if (vec && len % 512 == 0) {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crc8_warp_kernel<0>, kCrcWarpBlock,
-                                                  0);
+  // Which kernel.  Measured, 2^20 messages, P = 0x1D (us; in brackets 20,000):
+  //   length              28        60        100       140       1000
+  //   table, a thread     17 (11)   46 (11)   116 (12)  246 (14)  -
+  //   warp, units         140 (15)  141 (16)  147 (16)  150 (16)  256
+  //   length, aligned     32        64        128       160       208      1008
+  //   cp.async tiles      25 (13)   42 (20)   83 (35)   110 (41)  170 (55) 724
+  //   warp, units         120 (15)  120 (16)  125 (15)  126 (15)  127 (16) 238
+  // (bitsliced by a thread per 32 messages, which these replace: 258 for 60
+  // bytes, 4212 for 1000, 2743 for 10,000 messages of 1500.)  The warp kernel
+  // spends about 110 on every 512-byte chunk, or part of one, of 2^20 messages;
+  // the tiles need enough messages to fill the chip.
+  const bool whole = vec && len % 512 == 0;
+  const bool tiles = vec && len > 32 && len <= 160 && n >= (size_t(1) << 19);
+  if (whole || (len > 112 && !tiles)) {
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crc8_warp_kernel<0, false>,
+                                                  kCrcWarpBlock, 0);
     const size_t G = (n + 31) / 32;
     const size_t blocks = (G + kCrcWarpBlock / 32 - 1) / (kCrcWarpBlock / 32);
     const uint32_t grid = uint32_t(std::min<size_t>(blocks, size_t(sms) * std::max(per_sm, 1)));
-    const CrcJoin cj = crc_join_matrices(poly);
-    switch (poly) {
-      case 0x07: launch_crc_warp<0x07>(grid, st, d_data, n, len, poly, init, xorout, d_crc, cj, G); break;
-      case 0x1D: launch_crc_warp<0x1D>(grid, st, d_data, n, len, poly, init, xorout, d_crc, cj, G); break;
-      case 0x2F: launch_crc_warp<0x2F>(grid, st, d_data, n, len, poly, init, xorout, d_crc, cj, G); break;
-      case 0x31: launch_crc_warp<0x31>(grid, st, d_data, n, len, poly, init, xorout, d_crc, cj, G); break;
-      case 0x9B: launch_crc_warp<0x9B>(grid, st, d_data, n, len, poly, init, xorout, d_crc, cj, G); break;
-      case 0xD5: launch_crc_warp<0xD5>(grid, st, d_data, n, len, poly, init, xorout, d_crc, cj, G); break;
-      default: launch_crc_warp<0>(grid, st, d_data, n, len, poly, init, xorout, d_crc, cj, G);
-    }
-  } else if (vec) {
+    launch_crc_warp(poly, !whole, grid, st, d_data, n, len, poly, init, xorout, d_crc,
+                    crc_join_matrices(poly), crc_past(poly, len), G);
+  } else if (tiles) {
     if (cudaFuncSetAttribute(crc8_async_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              int(kCrcTileBytes)) != cudaSuccess)
       return set_error(MICKEY_E_CUDA, "crc kernel shared memory");
@@ -697,12 +738,11 @@ MICKEY_API int mickey_crc8(const uint8_t *data, size_t n, size_t len, uint8_t po
     crc8_async_kernel<<<uint32_t(grid), kCrcGroups, kCrcTileBytes, st>>>(
         d_data, n, len, poly, init, xorout, d_crc, n_tiles);
   } else {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crc8_regs_kernel, kCrcThreads, 0);
-    const size_t G = (n + 31) / 32;
-    const size_t blocks = (G + kCrcThreads - 1) / kCrcThreads;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crc8_table_kernel, kCrcTableThreads, 0);
+    const size_t blocks = (n + kCrcTableThreads - 1) / kCrcTableThreads;
     const size_t grid = std::min<size_t>(blocks, size_t(sms) * std::max(per_sm, 1));
-    crc8_regs_kernel<<<uint32_t(grid), kCrcThreads, 0, st>>>(d_data, n, len, poly, init, xorout,
-                                                             d_crc, false, G);
+    crc8_table_kernel<<<uint32_t(grid), kCrcTableThreads, 0, st>>>(d_data, n, len, poly, init,
+                                                                   xorout, d_crc);
   }
   if (cudaGetLastError() != cudaSuccess) return set_error(MICKEY_E_CUDA, "crc kernel launch");
   if (mem == MICKEY_MEM_HOST) {

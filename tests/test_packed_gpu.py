@@ -286,3 +286,25 @@ def test_ragged_thread_per_group_and_per_instance_agree(monkeypatch, n, layout):
         bits = np.unpackbits(np.asarray(want[k]))[lo:lo + 64]
         assert np.array_equal(np.packbits(bits), nxt[0][k])
         assert np.array_equal(nxt[0][k], nxt[1][k])
+
+
+# the covering units: first and last unit in one, one chunk to several, every
+# alignment of data and length, the edges of the buffer, presets of 0 and not
+@pytest.mark.parametrize("length", [25, 26, 31, 33, 47, 161, 176, 481, 482, 497, 498, 511, 513, 528,
+                                    1000, 1009, 1536 + 7])
+@pytest.mark.parametrize("poly,init,xorout", [(0x1D, 0xFF, 0xFF), (0x07, 0, 0), (0x55, 0xA5, 0x3C),
+                                              (0x32, 0xFF, 0)])
+def test_crc8_any_length_and_alignment(length, poly, init, xorout):
+    from oracle import lfsr as ol
+    from paper_1909_04750_gb300.lfsr import crc8
+    for n in (1, 31, 33, 150):
+        raw = np.random.default_rng(length + n).integers(0, 256, n * length).astype(np.uint8)
+        want = ol.crc8_batch(raw.reshape(n, length), poly, init, xorout)
+        for offset in (0, 1, 8, 15):
+            buf = torch.zeros(n * length + 16, dtype=torch.uint8, device="cuda")
+            buf[offset:offset + n * length] = torch.from_numpy(raw).cuda()
+            buf[:offset] = 0xC3
+            buf[offset + n * length:] = 0xC3
+            data = buf[offset:offset + n * length].view(n, length)
+            got = crc8(data, poly, init, xorout).cpu().numpy()
+            assert np.array_equal(got, want), (n, offset)
