@@ -214,9 +214,11 @@ MICKEY_API mickey_streams *mickey_import_state(const uint8_t *states,
  *           MICKEY_MODE_PERSISTENT2: two warps per SM sub-partition, each
  *           clocking and emitting (two blocks per SM, rows staged four
  *           tiles deep; with too few warp-groups it runs as PERSISTENT);
- *           MICKEY_MODE_AUTO: one thread per instance for handles of up to 52
- *           32-lane groups per SM (about 250,000 instances; unroll and stage
- *           have no effect there), else as PERSISTENT.
+ *           MICKEY_MODE_AUTO: one thread per instance for handles of up to 18
+ *           32-lane groups per SM (about 87,000 instances; up to 52 for rows of
+ *           bytes that are not whole words), four warps per 32 groups for
+ *           handles of up to 96 groups per SM (about 467,000 instances), else
+ *           as PERSISTENT; unroll and stage only matter there.
  *   unroll  clocks per inner step, 2 or 4.
  *   stage   the output tile of the row layouts: 0 writes each 32-clock tile's
  *           4 bytes per row directly; otherwise each row's words of several

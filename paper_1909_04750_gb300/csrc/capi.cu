@@ -207,9 +207,16 @@ int allocate(mickey_streams *s, size_t n) {
   return ok();
 }
 
-// Whether launches left to the library clock one instance per thread.
+// Whether initialisations and ragged calls left to the library clock one
+// instance per thread.
 bool use_packed(const mickey_streams *s) {
   return s->G <= kPackedPerSm * uint32_t(s->sm_count);
+}
+
+// Whether launches left to the library take four warps per warp-group when
+// they do not clock one instance per thread.
+bool use_quarters(const mickey_streams *s) {
+  return (s->G + 31) / 32 <= kQuartersPerSm * uint32_t(s->sm_count);
 }
 
 // Key/IV loading + preclock for all instances of s.
@@ -305,7 +312,7 @@ void set_hand_off(mickey_streams *s, PersistArgs &pa) {
 }
 
 // One keystream launch of `bits` clocks into a device buffer.
-//   AUTO, few groups          one thread per instance
+//   AUTO, few groups          one thread per instance, or four warps per warp-group
 //   GRID                      one thread per group, clocking and emitting
 //   PERSISTENT2, enough groups two clocking warps per SM sub-partition
 //   otherwise (AUTO, PERSISTENT) the paired kernel: clock warps beside emission
@@ -319,9 +326,18 @@ int launch_generate(mickey_streams *s, uint64_t bits, void *out, int layout) {
   int mode = c.set ? c.mode : s->mode;
   const int unroll = c.set ? c.unroll : s->unroll;
   const int stage = c.set ? c.stage : s->stage;
-  if (mode == MICKEY_MODE_AUTO && use_packed(s)) {
-    CUDA_TRY(launch_packed_keystream(ka, layout, s->stream), "packed_keystream_kernel launch");
-    return MICKEY_OK;
+  if (mode == MICKEY_MODE_AUTO) {
+    const uint32_t sms = uint32_t(s->sm_count);
+    const bool words = layout != MICKEY_LAYOUT_BYTES ||
+                       ((bits + 7) / 8 % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 4 == 0);
+    if (s->G <= (words ? kPackedKeystreamPerSm : kPackedPerSm) * sms) {
+      CUDA_TRY(launch_packed_keystream(ka, layout, s->stream), "packed_keystream_kernel launch");
+      return MICKEY_OK;
+    }
+    if (use_quarters(s)) {
+      CUDA_TRY(launch_quarters(ka, layout, s->sm_count, s->stream), "quarters_kernel launch");
+      return MICKEY_OK;
+    }
   }
   if (mode == MICKEY_MODE_GRID) {
     CUDA_TRY(launch_keystream(ka, layout, unroll, stage, nullptr, s->stream),
@@ -812,7 +828,7 @@ int mickey_tune(mickey_streams *s, uint64_t n_bits, int layout, mickey_tune_resu
   for (int mode : {MICKEY_MODE_AUTO, MICKEY_MODE_GRID, MICKEY_MODE_PERSISTENT,
                    MICKEY_MODE_PERSISTENT2}) {
     if (mode == MICKEY_MODE_PERSISTENT2 && !use_persistent(s, mode)) continue;
-    if (mode == MICKEY_MODE_AUTO && !use_packed(s)) continue;   // else the same as PERSISTENT
+    if (mode == MICKEY_MODE_AUTO && !use_quarters(s)) continue;   // the same as PERSISTENT
     // output tile: direct row stores, or rows staged this many tiles deep
     // (the depths the mode's kernels are compiled for)
     std::vector<int> stages{mode == MICKEY_MODE_AUTO ? 1 : 0};
@@ -824,7 +840,7 @@ int mickey_tune(mickey_streams *s, uint64_t n_bits, int layout, mickey_tune_resu
         if (n_bits % (32 * uint64_t(d)) == 0) stages.push_back(d);
     }
     for (int unroll : kUnrolls) {
-      if (mode == MICKEY_MODE_AUTO && unroll != 4) continue;      // the packed launch has no choice
+      if (mode == MICKEY_MODE_AUTO && unroll != 4) continue;      // its own launches have no choice
       for (int stage : stages) {
         auto &c = s->cfg[layout];
         c.set = true;

@@ -49,15 +49,19 @@ cudaError_t launch_init(const LoadArgs &a, uint32_t *state, cudaStream_t st);
 cudaError_t launch_packed_init(const LoadArgs &a, uint32_t *state, cudaStream_t st);
 
 // Launches of a handle whose mode is left to the library take one thread per
-// instance up to this many groups per SM, one thread per 32-lane group above.
-// Measured (152 SMs, us for 2048 bits of bytes / of a re-key; packed, thread
-// per group):
-//   groups    608      2432     4864     7296     8512
-//   2048 bits 76, 712  216, 710 412, 713 606, 713 703, 712
-//   re-key    30, 118  50, 119  77, 120  106, 120 121, 119
+// instance up to this many groups per SM.  Measured (152 SMs, us; 2048 bits of
+// bytes: packed, four warps per warp-group, thread per group; re-key: packed,
+// thread per group):
+//   groups    608       2432           4864           7296           9728
+//   2048 bits 69, -, 712 212, 240, 711 407, 240, 713  604, 385, 713  -, 385, 713
+//   re-key    27, 118   49, 119        77, 119        108, 119       136, 120
 // The packed times grow with the groups once every SM sub-partition has a
-// warp; a thread per group takes the time of one group's chain until all 608
-// sub-partitions have a warp of 32 groups (19456 groups), so the lines cross.
+// warp; four warps take a warp-group's clock in 117 ns with one per SM, 187
+// with two, 270 with three; a thread per group takes 334 ns until all 608
+// sub-partitions have a warp of 32 groups.  Rows of bytes that are not whole
+// words cost the emission warps byte stores: there the packed launch goes as
+// far as it beats a thread per group.
+constexpr uint32_t kPackedKeystreamPerSm = 18;
 constexpr uint32_t kPackedPerSm = 52;
 
 struct KeystreamArgs {
@@ -127,6 +131,12 @@ cudaError_t launch_ragged(const RaggedArgs &a, int layout, const PersistArgs *p,
 // One thread per instance (packed.cu), any n_bits, layout and alignment that
 // launch_keystream takes.
 cudaError_t launch_packed_keystream(const KeystreamArgs &a, int layout, cudaStream_t st);
+
+// Four warps per warp-group (keystream_quarters.cu), at most kQuartersPerSm
+// warp-groups per SM; any n_bits, layout and alignment that launch_keystream
+// takes.
+constexpr uint32_t kQuartersPerSm = 3;
+cudaError_t launch_quarters(const KeystreamArgs &a, int layout, int sm_count, cudaStream_t st);
 
 // Grain with one thread per instance (grain_packed.cu): the bitsliced or the
 // bytes layout, any n_bits and alignment that grain_generate takes; loading and

@@ -78,19 +78,28 @@ def test_output_at_any_alignment(n_bits, offset):
     assert (got[:offset] == 0xA5).all() and (got[offset + want.size:] == 0xA5).all()
 
 
+# the last groups per SM of the packed launch, of one and two warp-groups per
+# SM, of the packed initialisation, of three warp-groups, and one group more
 @pytest.mark.parametrize("extra", [0, 1])
-def test_last_size_and_the_next_agree_with_a_thread_per_group(monkeypatch, extra):
-    # the largest handle of the packed launches and one group more, against an
-    # explicit grid launch: output, a second call, the state
+@pytest.mark.parametrize("per_sm", [18, 32, 52, 64, 96])
+def test_last_size_and_the_next_agree_with_a_thread_per_group(monkeypatch, per_sm, extra):
+    # against an explicit grid launch: output, calls that go on, the state
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    s = _mixed((52 * sms + extra) * 32 - 5)
+    s = _mixed((per_sm * sms + extra) * 32 - 5)
     auto = _streams(s)
     monkeypatch.setenv("MICKEY_MODE", "grid")
     grid = _streams(s)
-    for n_bits, layout in ((64, "bytes"), (96, "u32"), (33, "bitsliced")):
+    for n_bits, layout in ((64, "bytes"), (96, "u32"), (33, "bitsliced"), (544, "bytes"),
+                           (1, "bytes"), (256, "u32_f32"), (45, "bytes"), (100, "bitsliced")):
         assert torch.equal(auto.generate(n_bits, layout), grid.generate(n_bits, layout))
-    states = [h.export_state()[0] for h in (auto, grid)]
-    assert np.array_equal(*states)
+    out = torch.zeros(s.n * 8 + 3, dtype=torch.uint8, device="cuda")   # off the word grid
+    got = auto.generate(64, "bytes", out=out[3:])
+    assert torch.equal(got.view(s.n, 8), grid.generate(64, "bytes"))
+    assert torch.equal(auto.generate(96, "bytes"), grid.generate(96, "bytes"))
+    k = 20_000
+    if extra == 0 and per_sm in (18, 32):
+        states = [h.export_state()[0][:k] for h in (auto, grid)]
+        assert np.array_equal(*states)
 
 
 @pytest.mark.parametrize("n", [32 * 300 + 7, 5 * 1024 + 1])
