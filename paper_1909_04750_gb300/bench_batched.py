@@ -50,7 +50,8 @@ def lone_split_ns_per_clock(n_bits: int = 1 << 18) -> float:
 
 
 def lone_group_ns_per_clock(n_bits: int = 1 << 16) -> float:
-    """Time per clock of one 32-lane group alone on the GPU."""
+    """Time per clock of one 32-lane group alone on the GPU, as a streams handle
+    runs it (a thread per instance)."""
     s = workloads.plain_scale(32)
     st = Streams(torch.from_numpy(s.keys).cuda(), torch.from_numpy(s.ivs).cuda())
     out = st.generate(n_bits, "bitsliced")

@@ -301,9 +301,9 @@ constexpr double kPackedNs[4] = {29.0, 52.0, 76.0, 100.0};
 // clocks 32 groups at 820 ns per clock (1140 when two share a sub-partition),
 // so it wins only once there are items for every warp and their lengths are
 // alike.  Measured, all split against the best of no split (ms): 20,000
-// streams of 2^10..2^18 bits 8.6, 158; 100,000 of 2^10..2^22 138, 2860;
+// streams of 2^10..2^18 bits 7.0, 158; 100,000 of 2^10..2^22 109, 2860;
 // 700,000 of 2^13 7.57, 9.99; 1.5 M of 2^12 8.32, 8.95; 4 M of 2^10..2^13
-// 18.5, 17.9.
+// 18.5, 17.9 (the last three with a packed clock 10 % slower than now).
 constexpr uint32_t kSplitAllPerSm = 400;
 
 // The arrangement of a new plan: all groups split, with as many warps per SM

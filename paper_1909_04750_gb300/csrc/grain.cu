@@ -156,7 +156,6 @@ struct grain_streams {
   uint32_t *d_state = nullptr;
   uint8_t *d_inputs = nullptr;   // host inputs staged: keys (10n), ivs (8n)
   uint32_t *d_flags = nullptr;   // one word per warp-group (hand-off between segments)
-  uint32_t epoch = 0;
   int *d_err = nullptr;
   cudaStream_t stream = nullptr;
   uint64_t pos = 0;
@@ -239,7 +238,6 @@ MICKEY_API grain_streams *grain_init_streams(const void *keys, const void *ivs, 
                 cudaSuccess &&
             cudaMalloc(&s->d_state, size_t(2 * kG) * s->Gpad * 4) == cudaSuccess &&
             cudaMalloc(&s->d_flags, size_t(s->Gpad / 32) * 4) == cudaSuccess &&
-            cudaMemsetAsync(s->d_flags, 0, size_t(s->Gpad / 32) * 4, s->stream) == cudaSuccess &&
             cudaMalloc(&s->d_err, sizeof(int)) == cudaSuccess &&
             cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream) == cudaSuccess;
   if (const char *v = getenv("MICKEY_SPIN_LIMIT")) {
@@ -323,8 +321,11 @@ MICKEY_API int grain_generate(grain_streams *s, uint64_t n_bits, void *out, int 
   pa.W = uint32_t(W);
   pa.L = (W * NT + slots - 1) / slots;
   pa.flags = s->d_flags;
-  s->epoch = s->epoch % 0x7fffffffu + 1;
-  pa.epoch = pa.wait_epoch = s->epoch;
+  pa.epoch = pa.wait_epoch = 1;
+  // the flags are cleared on the stream, not told apart by a count of calls,
+  // so that a captured call can be replayed
+  if (pa.cooperative && cudaMemsetAsync(s->d_flags, 0, size_t(W) * 4, s->stream) != cudaSuccess)
+    return grain_fail(MICKEY_E_CUDA, "flag reset");
   pa.spin_limit = s->spin_limit;
   pa.err = s->d_err;
   pa.tails_first = hand_off;

@@ -317,3 +317,25 @@ def test_crc8_any_length_and_alignment(length, poly, init, xorout):
             data = buf[offset:offset + n * length].view(n, length)
             got = crc8(data, poly, init, xorout).cpu().numpy()
             assert np.array_equal(got, want), (n, offset)
+
+
+def test_grain_hand_offs_in_a_replayed_graph(monkeypatch):
+    # a captured call whose segments hand states on, replayed three times,
+    # continues the streams as three calls do
+    monkeypatch.setenv("MICKEY_GRAIN_QUEUE", "1")
+    s = workloads.grain_streams(3 * 1024 + 17, seed=25)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        st = _grain(s)
+        out = torch.zeros((s.n, 64), dtype=torch.uint8, device="cuda")
+        st.generate(512, "bytes", out=out)
+        side.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            st.generate(512, "bytes", out=out)
+    plain = _grain(s)
+    plain.generate(512, "bytes")
+    for _ in range(3):
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, plain.generate(512, "bytes"))
