@@ -40,7 +40,7 @@ WORKLOAD = ("plain_scale: 2^20 MICKEY 2.0 instances (32768 bitsliced groups), 80
 # digest) and that launch with its row staging (the unroll depth does not
 # change what is written; 4-tile staging moved 6.13 GB); otherwise traffic
 # is null.
-KEYSTREAM_TRAFFIC = {"digest": "9ad179c176d46a4f", "launch": ("persistent, ", " staged rows"),
+KEYSTREAM_TRAFFIC = {"digest": "1796d74fd0592389", "launch": ("persistent, ", " staged rows"),
                      "bytes_per_launch": 2275865856}
 
 
