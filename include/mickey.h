@@ -237,7 +237,10 @@ MICKEY_API mickey_streams *mickey_import_state(const uint8_t *states,
  * MICKEY_E_TIMEOUT and that call's output and state are undefined;
  * MICKEY_TEST_UNPUBLISHED=1 is a test hook that makes every such wait run
  * out (tails wait for a value no head writes), to exercise that path
- * without a fault.
+ * without a fault; MICKEY_TEST_TAILS_FIRST=1 one that makes every segment of a
+ * keystream launch wait for the one before it.  A captured mickey_generate
+ * can be replayed: each replay continues the streams as a call does, except
+ * that mickey_position does not see it.
  * ------------------------------------------------------------------------ */
 #define MICKEY_MODE_AUTO 0
 #define MICKEY_MODE_GRID 1

@@ -36,10 +36,10 @@ struct mickey_streams {
   } cfg[4];                       // per-layout settings (mickey_set_config / tune)
   int sm_count = 0;
   int persist_blocks = 0;         // blocks of the persistent kernel (<= SMs)
-  uint32_t *d_flags = nullptr;    // persistent mode: one word per warp-group
-  uint32_t epoch = 0;
+  uint32_t *d_flags = nullptr;    // one word per warp-group (hand-off between segments)
   uint32_t spin_limit = 1u << 24;   // polls of ~256 ns before a tail piece gives up
   bool test_unpublished = false;    // test hook: tails wait for a value no head writes
+  bool test_tails_first = false;    // test hook: every hand-off is waited for
   // Keystream position of stream i = pos_base + pos[i]: a call that
   // continues every stream by the same count moves pos_base only (O(1) host
   // work, whatever n is); ragged calls and imports set pos[i]; pos_max is
@@ -187,6 +187,7 @@ int allocate(mickey_streams *s, size_t n) {
     if (l > 0 && l < (1ll << 31)) s->spin_limit = uint32_t(l);
   }
   if (const char *v = getenv("MICKEY_TEST_UNPUBLISHED")) s->test_unpublished = atoi(v) != 0;
+  if (const char *v = getenv("MICKEY_TEST_TAILS_FIRST")) s->test_tails_first = atoi(v) != 0;
   int dev = 0;
   CUDA_TRY(cudaGetDevice(&dev), "cudaGetDevice");
   CUDA_TRY(cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, dev),
@@ -197,8 +198,6 @@ int allocate(mickey_streams *s, size_t n) {
     if (b > 0 && b < s->sm_count) s->persist_blocks = b;
   }
   CUDA_TRY(cudaMalloc(&s->d_flags, size_t((s->G + 31) / 32) * 4), "cudaMalloc(flags)");
-  CUDA_TRY(cudaMemsetAsync(s->d_flags, 0, size_t((s->G + 31) / 32) * 4, s->stream),
-           "cudaMemset(flags)");
   CUDA_TRY(cudaMalloc(&s->d_state, size_t(kStateRows) * s->Gpad * 4), "cudaMalloc(state)");
   CUDA_TRY(cudaMalloc(&s->d_scratch, size_t(kScratchRows + 1) * s->Gpad * 4),
            "cudaMalloc(scratch)");
@@ -300,15 +299,18 @@ bool use_persistent(const mickey_streams *s, int mode) {
   return mode != MICKEY_MODE_GRID && W >= slots;
 }
 
-// The flags and the epoch that the segments of one launch hand states on with.
-void set_hand_off(mickey_streams *s, PersistArgs &pa) {
+// What the segments of one launch hand states on with.  The flags are cleared
+// on the stream before a launch that uses them, not told apart by a count of
+// calls, so that a captured call can be replayed.
+cudaError_t set_hand_off(mickey_streams *s, PersistArgs &pa) {
   pa.flags = s->d_flags;
-  s->epoch = s->epoch % 0x7fffffffu + 1;   // 1 .. 2^31 - 1 (0 is the flags' initial value)
-  pa.epoch = s->epoch;
-  pa.wait_epoch = s->test_unpublished ? (s->epoch | 0x80000000u) : s->epoch;
+  pa.epoch = 1;
+  pa.wait_epoch = s->test_unpublished ? 2 : 1;
   pa.spin_limit = s->spin_limit;
   pa.err = s->d_err;
-  pa.tails_first = 0;
+  pa.tails_first = s->test_tails_first;
+  return pa.cooperative ? cudaMemsetAsync(s->d_flags, 0, size_t(pa.W) * 4, s->stream)
+                        : cudaSuccess;
 }
 
 // One keystream launch of `bits` clocks into a device buffer.
@@ -362,7 +364,7 @@ int launch_generate(mickey_streams *s, uint64_t bits, void *out, int layout) {
     pa.cooperative = 0;
     pa.L = NT;
   }
-  set_hand_off(s, pa);
+  CUDA_TRY(set_hand_off(s, pa), "cudaMemset(flags)");
   CUDA_TRY(launch_keystream(ka, layout, unroll, stage, &pa, s->stream),
            "keystream persistent launch");
   return MICKEY_OK;
@@ -590,7 +592,7 @@ int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
   pa.cooperative = slots < W;
   pa.W = uint32_t(W);
   pa.L = std::max(longest, (blocks[W] + slots - 1) / slots);
-  set_hand_off(s, pa);
+  if (!packed) CUDA_TRY(set_hand_off(s, pa), "cudaMemset(flags)");
   CUDA_TRY(launch_ragged(ra, layout, packed ? nullptr : &pa, s->stream), "ragged launch");
   CUDA_TRY(cudaEventRecord(s->ev_ragged, s->stream), "record");
   for (size_t i = 0; i < n; ++i) {

@@ -90,7 +90,7 @@ constexpr uint64_t kMaxBitsPerCall = 1ull << 34;
 constexpr int kKsThreads = 128;
 
 // Persistent mode (see keystream_persistent_kernel): W warp-groups, L tiles
-// per warp, one flag word per warp-group (compared with `epoch`).
+// per warp, one flag word per warp-group, zero before a cooperative launch.
 struct PersistArgs {
   uint32_t blocks;      // grid: 1 or 2 blocks per SM (cooperative), or one block per
                         // 4 warp-groups (paired launch with L = NT, not cooperative)
