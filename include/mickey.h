@@ -160,7 +160,9 @@ MICKEY_API size_t mickey_output_bytes(size_t n, uint64_t n_bits, int layout);
  * position moves): MICKEY_E_ARG (NULL pointer, a length above 2^34, a
  * misaligned 32-bit output), MICKEY_E_LAYOUT (MICKEY_LAYOUT_U32_F32, or a
  * u32 length not a multiple of 32), MICKEY_E_LIMIT (a stream would pass 2^40
- * bits), MICKEY_E_OOM / MICKEY_E_CUDA.
+ * bits), MICKEY_E_OOM / MICKEY_E_CUDA.  As after mickey_generate, mickey_sync
+ * reports MICKEY_E_TIMEOUT should a hand-off between warps not come
+ * (MICKEY_SPIN_LIMIT polls, and one more per clock of a warp's share).
  * ------------------------------------------------------------------------ */
 MICKEY_API int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
                                       const uint64_t *out_offsets, int layout);

@@ -537,8 +537,8 @@ int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
   // The lengths and offsets reach the kernel through one of two pinned
   // buffers (so that the copy is a DMA and the next call can fill the other
   // buffer while this one is in flight) and one device buffer.
-  // ... then the prefix sums of the warp-groups' blocks
-  const size_t W = (G + 31) / 32, words = n + n_off + W + 1;
+  // ... then, for the launch with a thread per group, its work line
+  const size_t W = (G + 31) / 32, words = n + n_off + 2 * W + 1;
   if (s->ragged_words < words) {
     if (s->ev_ragged) CUDA_TRY(cudaEventSynchronize(s->ev_ragged), "sync");
     for (int k = 0; k < 2; ++k) {
@@ -567,32 +567,43 @@ int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
     std::copy(out_offsets, out_offsets + n_off, h + n);
   else
     ragged_packed(n, n_bits, layout, h + n);
-  uint64_t *blocks = h + n + n_off, longest = 0;
-  blocks[0] = 0;
-  for (size_t w = 0; w < W; ++w) {
-    uint64_t c = 0;
-    for (size_t i = 1024 * w; i < std::min(n, 1024 * w + 1024); ++i) c = std::max(c, n_bits[i]);
-    c = (c + kRaggedBlockBits - 1) / kRaggedBlockBits;
-    blocks[w + 1] = blocks[w] + c;
-    longest = std::max(longest, c);
+  const auto &c = s->cfg[layout];
+  const bool packed = (c.set ? c.mode : s->mode) == MICKEY_MODE_AUTO && use_packed(s);
+  const uint64_t slots = std::min<uint64_t>(W, 4ull * uint32_t(s->persist_blocks));
+  RaggedLine line{};
+  if (!packed) {
+    std::vector<uint64_t> blocks(W, 0);
+    for (size_t w = 0; w < W; ++w) {
+      for (size_t i = 1024 * w; i < std::min(n, 1024 * w + 1024); ++i)
+        blocks[w] = std::max(blocks[w], n_bits[i]);
+      blocks[w] = (blocks[w] + kRaggedBlockBits - 1) / kRaggedBlockBits;
+    }
+    uint64_t *order = h + n + n_off;
+    line = ragged_cuts(blocks.data(), uint32_t(W), slots, order, order + W);
+    line.order = s->d_ragged + n + n_off;    // where the copy below puts them
+    line.blocks = line.order + W;
   }
   // the previous ragged launch (perhaps on another stream) has read d_ragged
   CUDA_TRY(cudaStreamWaitEvent(s->stream, s->ev_ragged, 0), "wait");
-  CUDA_TRY(cudaMemcpyAsync(s->d_ragged, h, words * 8, cudaMemcpyHostToDevice, s->stream),
+  CUDA_TRY(cudaMemcpyAsync(s->d_ragged, h, (packed ? n + n_off : words) * 8,
+                           cudaMemcpyHostToDevice, s->stream),
            "H2D ragged lengths");
   CUDA_TRY(cudaEventRecord(s->ev_h2d[kb], s->stream), "record");
   s->ragged_flip = kb ^ 1;
   RaggedArgs ra{s->d_state, s->G, s->Gpad, n, s->d_ragged, s->d_ragged + n,
-                static_cast<uint8_t *>(out), s->d_ragged + n + n_off};
-  const auto &c = s->cfg[layout];
-  const bool packed = (c.set ? c.mode : s->mode) == MICKEY_MODE_AUTO && use_packed(s);
-  const uint64_t slots = std::min<uint64_t>(W, 4ull * uint32_t(s->persist_blocks));
+                static_cast<uint8_t *>(out), line};
   PersistArgs pa{};
   pa.blocks = uint32_t((slots + 3) / 4);
-  pa.cooperative = slots < W;
+  pa.cooperative = line.alone < W;
   pa.W = uint32_t(W);
-  pa.L = std::max(longest, (blocks[W] + slots - 1) / slots);
-  if (!packed) CUDA_TRY(set_hand_off(s, pa), "cudaMemset(flags)");
+  if (!packed) {
+    CUDA_TRY(set_hand_off(s, pa), "cudaMemset(flags)");
+    // By the cuts a tail hardly waits.  The limit grows with the segments all
+    // the same: a warp whose rows cost it more stores may come to the hand-off
+    // a part of its segment later than the next one.
+    const uint64_t clocks = std::min<uint64_t>(line.L, ~0u / kRaggedBlockBits) * kRaggedBlockBits;
+    pa.spin_limit = uint32_t(std::min<uint64_t>(pa.spin_limit + clocks, ~0u));
+  }
   CUDA_TRY(launch_ragged(ra, layout, packed ? nullptr : &pa, s->stream), "ragged launch");
   CUDA_TRY(cudaEventRecord(s->ev_ragged, s->stream), "record");
   for (size_t i = 0; i < n; ++i) {

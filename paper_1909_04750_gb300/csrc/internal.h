@@ -7,6 +7,8 @@
 #include <cstddef>
 #include <cstdint>
 
+#include "ragged_cuts.h"
+
 namespace mickey {
 
 // Device-side error bits, OR-ed into a per-handle flag word.
@@ -119,13 +121,12 @@ struct RaggedArgs {
   const uint64_t *n_bits;   // n values, device
   const uint64_t *offsets;  // n (row layouts) or G (bitsliced) byte offsets, device
   uint8_t *out;
-  const uint64_t *blocks;   // W + 1 prefix sums of the warp-groups' blocks of
-                            // kRaggedBlockBits clocks (their longest lane's), device; only with `p`
+  RaggedLine line;          // the warp-groups in blocks of kRaggedBlockBits clocks (their
+                            // longest lane's), arrays on the device; only with `p`
 };
 constexpr uint32_t kRaggedBlockBits = 128;
 // p == nullptr: one thread per instance; else clock and emission warps on the
-// segments of the work line `blocks` (p->L blocks each, at least as many as any
-// warp-group has; p->cooperative = 0: warp-group w to clock warp w).
+// pieces of `line` (cooperative where it may be cut).
 cudaError_t launch_ragged(const RaggedArgs &a, int layout, const PersistArgs *p, cudaStream_t st);
 
 // One thread per instance (packed.cu), any n_bits, layout and alignment that

@@ -9,10 +9,8 @@
 // paired with emission warps as in the keystream launch
 // (keystream_persistent.cuh); a group is clocked as often as its longest lane
 // needs.  What differs from equal lengths:
-//   * The work line of warp-groups x blocks of 128 clocks has as many blocks
-//     per warp-group as its longest lane; segments are cut on the prefix sums,
-//     each at least as long as the longest warp-group, so that a warp-group
-//     spans two at most.
+//   * A warp-group has as many blocks of 128 clocks as its longest lane needs,
+//     and the work line is cut on their prefix sums (ragged_cuts.h).
 //   * A lane's state must be the one after exactly its own number of clocks.
 //     The clock loop has no test per clock: before every block the lanes that
 //     end within its 128 clocks are merged into the state in HBM
@@ -220,59 +218,6 @@ __device__ __forceinline__ void ragged_words(const RaggedArgs &a, const LaneTab 
   for (; c < n; ++c) o[c] = z[c * kKsThreads] & alive;
 }
 
-// The warp-group that holds block x of the work line: the last w with
-// blocks[w] <= x (x below blocks[W]).
-__device__ __forceinline__ uint32_t find_group(const uint64_t *blocks, uint32_t W, uint64_t x) {
-  uint32_t lo = 0, hi = W;
-  while (hi - lo > 1) {
-    const uint32_t mid = lo + (hi - lo) / 2;
-    if (blocks[mid] <= x) lo = mid;
-    else hi = mid;
-  }
-  return lo;
-}
-
-// Pieces of a segment in the order head, whole warp-groups, tail, as
-// segment_piece, on the prefix sums.  Without hand-offs (cooperative = 0)
-// slot w has warp-group w.
-__device__ __forceinline__ bool ragged_piece(const PersistArgs &p, const uint64_t *blocks,
-                                             uint32_t slot, uint32_t k, uint32_t &w, uint32_t &ta,
-                                             uint32_t &tb) {
-  if (!p.cooperative) {
-    w = slot;
-    ta = 0;
-    if (k || slot >= p.W) return false;
-    tb = kSnapTiles * uint32_t(blocks[slot + 1] - blocks[slot]);
-    return true;
-  }
-  const uint64_t total = blocks[p.W];
-  const uint64_t a = uint64_t(slot) * p.L, b = a + p.L < total ? a + p.L : total;
-  if (a >= b) return false;
-  const uint32_t wf = find_group(blocks, p.W, a), wl = find_group(blocks, p.W, b - 1);
-  const bool head = b < blocks[wl + 1] && (wl != wf || a == blocks[wf]);
-  if (head && k == 0) {
-    w = wl;
-    ta = 0;
-    tb = kSnapTiles * uint32_t(b - blocks[wl]);
-    return true;
-  }
-  k -= head ? 1 : 0;
-  const bool tail = a > blocks[wf];
-  const uint32_t lo = wf + (tail ? 1 : 0), hi = b < blocks[wl + 1] ? wl : wl + 1;   // whole: [lo, hi)
-  const uint32_t whole = hi > lo ? hi - lo : 0;
-  if (k < whole) {
-    w = lo + k;
-    ta = 0;
-    tb = kSnapTiles * uint32_t(blocks[w + 1] - blocks[w]);
-    return true;
-  }
-  if (k > whole || !tail) return false;
-  w = wf;
-  ta = kSnapTiles * uint32_t(a - blocks[wf]);
-  tb = kSnapTiles * uint32_t((b < blocks[wf + 1] ? b : blocks[wf + 1]) - blocks[wf]);
-  return true;
-}
-
 template <int LAYOUT>
 __global__ void __launch_bounds__(2 * kKsThreads, 1)
     ragged_ws_kernel(RaggedArgs a, PersistArgs p) {
@@ -287,11 +232,13 @@ __global__ void __launch_bounds__(2 * kKsThreads, 1)
   uint32_t par = 0;
 #pragma unroll 1
   for (uint32_t k = 0;; ++k) {
-    uint32_t w, ta, tb;
-    if (!ragged_piece(p, a.blocks, slot, k, w, ta, tb)) break;
-    if (ta == tb) continue;                  // a warp-group that asks for no bits
-    const uint32_t g = w * 32 + lane;
-    const bool ends = a.blocks[w] + tb / kSnapTiles == a.blocks[w + 1];
+    uint32_t pos;
+    uint64_t ba, bb;
+    if (!ragged_piece(a.line, p.tails_first, slot, k, pos, ba, bb)) break;
+    if (ba == bb) continue;                  // a warp-group that asks for no bits
+    const uint32_t w = uint32_t(a.line.order[pos]), g = w * 32 + lane;
+    const uint32_t ta = kSnapTiles * uint32_t(ba), tb = kSnapTiles * uint32_t(bb);
+    const bool ends = a.line.blocks[pos] + bb == a.line.blocks[pos + 1];
     if (clocker) {
       if (ta > 0) {  // tail: wait for the head piece of this warp-group
         uint32_t it = 0;
