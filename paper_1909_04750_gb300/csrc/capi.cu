@@ -198,6 +198,8 @@ int allocate(mickey_streams *s, size_t n) {
     if (b > 0 && b < s->sm_count) s->persist_blocks = b;
   }
   CUDA_TRY(cudaMalloc(&s->d_flags, size_t((s->G + 31) / 32) * 4), "cudaMalloc(flags)");
+  CUDA_TRY(cudaMemsetAsync(s->d_flags, 0, size_t((s->G + 31) / 32) * 4, s->stream),
+           "cudaMemset(flags)");
   CUDA_TRY(cudaMalloc(&s->d_state, size_t(kStateRows) * s->Gpad * 4), "cudaMalloc(state)");
   CUDA_TRY(cudaMalloc(&s->d_scratch, size_t(kScratchRows + 1) * s->Gpad * 4),
            "cudaMalloc(scratch)");
@@ -299,18 +301,13 @@ bool use_persistent(const mickey_streams *s, int mode) {
   return mode != MICKEY_MODE_GRID && W >= slots;
 }
 
-// What the segments of one launch hand states on with.  The flags are cleared
-// on the stream before a launch that uses them, not told apart by a count of
-// calls, so that a captured call can be replayed.
-cudaError_t set_hand_off(mickey_streams *s, PersistArgs &pa) {
+// What the segments of one launch hand states on with.
+void set_hand_off(const mickey_streams *s, PersistArgs &pa) {
   pa.flags = s->d_flags;
-  pa.epoch = 1;
-  pa.wait_epoch = s->test_unpublished ? 2 : 1;
+  pa.wait_flag = s->test_unpublished ? 2 : 1;
   pa.spin_limit = s->spin_limit;
   pa.err = s->d_err;
   pa.tails_first = s->test_tails_first;
-  return pa.cooperative ? cudaMemsetAsync(s->d_flags, 0, size_t(pa.W) * 4, s->stream)
-                        : cudaSuccess;
 }
 
 // One keystream launch of `bits` clocks into a device buffer.
@@ -364,7 +361,7 @@ int launch_generate(mickey_streams *s, uint64_t bits, void *out, int layout) {
     pa.cooperative = 0;
     pa.L = NT;
   }
-  CUDA_TRY(set_hand_off(s, pa), "cudaMemset(flags)");
+  set_hand_off(s, pa);
   CUDA_TRY(launch_keystream(ka, layout, unroll, stage, &pa, s->stream),
            "keystream persistent launch");
   return MICKEY_OK;
@@ -597,7 +594,7 @@ int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
   pa.cooperative = line.alone < W;
   pa.W = uint32_t(W);
   if (!packed) {
-    CUDA_TRY(set_hand_off(s, pa), "cudaMemset(flags)");
+    set_hand_off(s, pa);
     // By the cuts a tail hardly waits.  The limit grows with the segments all
     // the same: a warp whose rows cost it more stores may come to the hand-off
     // a part of its segment later than the next one.
@@ -701,6 +698,9 @@ int mickey_sync(mickey_streams *s) {
   CUDA_TRY(cudaMemcpy(&flag, s->d_err, sizeof flag, cudaMemcpyDeviceToHost), "D2H err");
   if (flag) {
     CUDA_TRY(cudaMemset(s->d_err, 0, sizeof(int)), "clear err");
+    if (flag & kErrTimeout)   // the hand-offs that nobody waited for any more
+      CUDA_TRY(cudaMemsetAsync(s->d_flags, 0, size_t((s->G + 31) / 32) * 4, s->stream),
+               "clear flags");
     if (flag & kErrIvLen) return fail(MICKEY_E_IVLEN, "an IV length above 80 bits was given");
     if (flag & kErrTimeout) return fail(MICKEY_E_TIMEOUT, "a device-side wait timed out");
   }

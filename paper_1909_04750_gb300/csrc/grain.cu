@@ -239,6 +239,7 @@ MICKEY_API grain_streams *grain_init_streams(const void *keys, const void *ivs, 
             cudaMalloc(&s->d_state, size_t(2 * kG) * s->Gpad * 4) == cudaSuccess &&
             cudaMalloc(&s->d_flags, size_t(s->Gpad / 32) * 4) == cudaSuccess &&
             cudaMalloc(&s->d_err, sizeof(int)) == cudaSuccess &&
+            cudaMemsetAsync(s->d_flags, 0, size_t(s->Gpad / 32) * 4, s->stream) == cudaSuccess &&
             cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream) == cudaSuccess;
   if (const char *v = getenv("MICKEY_SPIN_LIMIT")) {
     const long long l = atoll(v);
@@ -321,11 +322,7 @@ MICKEY_API int grain_generate(grain_streams *s, uint64_t n_bits, void *out, int 
   pa.W = uint32_t(W);
   pa.L = (W * NT + slots - 1) / slots;
   pa.flags = s->d_flags;
-  pa.epoch = pa.wait_epoch = 1;
-  // the flags are cleared on the stream, not told apart by a count of calls,
-  // so that a captured call can be replayed
-  if (pa.cooperative && cudaMemsetAsync(s->d_flags, 0, size_t(W) * 4, s->stream) != cudaSuccess)
-    return grain_fail(MICKEY_E_CUDA, "flag reset");
+  pa.wait_flag = 1;
   pa.spin_limit = s->spin_limit;
   pa.err = s->d_err;
   pa.tails_first = hand_off;
@@ -354,6 +351,8 @@ MICKEY_API int grain_sync(grain_streams *s) {
     return grain_fail(MICKEY_E_CUDA, "error flag copy");
   if (flag) {
     cudaMemset(s->d_err, 0, sizeof(int));
+    // the hand-offs that nobody waited for any more
+    cudaMemsetAsync(s->d_flags, 0, size_t(s->Gpad / 32) * 4, s->stream);
     return grain_fail(MICKEY_E_TIMEOUT, "a device-side wait timed out");
   }
   return set_error(MICKEY_OK, "");

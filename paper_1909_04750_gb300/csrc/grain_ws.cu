@@ -177,24 +177,9 @@ __global__ void __launch_bounds__(2 * kKsThreads, 1)
     if (!segment_piece(p, NT, slot, k, w, ta, tb)) break;
     const uint32_t g = w * 32 + lane;
     if (threadIdx.x < kKsThreads) {
-      if (ta > 0) {  // tail: wait for the head piece of this warp-group
-        uint32_t it = 0;
-        bool ok = true;
-        while (load_acquire(p.flags + w) != p.wait_epoch) {
-          if (++it > p.spin_limit) {
-            ok = false;
-            break;
-          }
-          __nanosleep(256);
-        }
-        if (!__all_sync(0xffffffffu, ok) && lane == 0) atomicOr(p.err, kErrTimeout);
-      }
+      if (ta > 0) await_head(p, w, lane);
       grain_clock_piece<LAYOUT>(a, g, zb0, zb1, par, 1 + pair, ta, tb);
-      if (ta == 0 && tb < NT) {  // head: publish the state for the next segment
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) store_release(p.flags + w, p.epoch);
-      }
+      if (ta == 0 && tb < NT) publish_head(p, w, lane);
     } else if (LAYOUT == kLayoutBytesLsb && e.stage) {
       grain_emit_rows(a, g, zb0, zb1, zs + kTileBufWords + t, par, 1 + pair, ta, tb,
                       g == a.G - 1 ? e.lane_mask : ~0u);

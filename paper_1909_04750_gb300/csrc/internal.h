@@ -92,7 +92,8 @@ constexpr uint64_t kMaxBitsPerCall = 1ull << 34;
 constexpr int kKsThreads = 128;
 
 // Persistent mode (see keystream_persistent_kernel): W warp-groups, L tiles
-// per warp, one flag word per warp-group, zero before a cooperative launch.
+// per warp, one flag word per warp-group: zero before a cooperative launch, 1
+// from the end of a head piece until its tail piece has seen it, zero after it.
 struct PersistArgs {
   uint32_t blocks;      // grid: 1 or 2 blocks per SM (cooperative), or one block per
                         // 4 warp-groups (paired launch with L = NT, not cooperative)
@@ -102,8 +103,7 @@ struct PersistArgs {
   uint32_t W;           // warp-groups = ceil(G / 32)
   uint64_t L;           // tiles of the work line per warp
   uint32_t *flags;      // W words
-  uint32_t epoch;       // value a finished head piece writes
-  uint32_t wait_epoch;  // value a tail piece waits for (== epoch; differs only under the
+  uint32_t wait_flag;   // value a tail piece waits for (1; differs only under the
                         // MICKEY_TEST_UNPUBLISHED test hook, to make the wait run out)
   uint32_t spin_limit;  // bounded wait of a tail piece (iterations of ~256 ns)
   int *err;

@@ -17,6 +17,36 @@ __device__ __forceinline__ void store_release(uint32_t *p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// The bounded wait of a tail piece (the whole warp) for the head of its
+// warp-group.  The flag is taken back at once, so the flags are zero again when
+// the launch ends: nothing clears them between calls, and a captured call can
+// be replayed.  When the wait runs out the error flag is raised, and the flag,
+// which the head may still set, stays; the call that reports the error clears
+// them all.
+__device__ __forceinline__ bool await_head(const PersistArgs &p, uint32_t w, uint32_t lane) {
+  uint32_t it = 0;
+  bool ok = true;
+  while (load_acquire(p.flags + w) != p.wait_flag) {
+    if (++it > p.spin_limit) {
+      ok = false;
+      break;
+    }
+    __nanosleep(256);
+  }
+  ok = __all_sync(0xffffffffu, ok);
+  if (lane == 0) {
+    if (ok) *reinterpret_cast<volatile uint32_t *>(p.flags + w) = 0u;
+    else atomicOr(p.err, kErrTimeout);
+  }
+  return ok;
+}
+// The end of a head piece: the warp's stores of the state, then the flag.
+__device__ __forceinline__ void publish_head(const PersistArgs &p, uint32_t w, uint32_t lane) {
+  __threadfence();
+  __syncwarp();
+  if (lane == 0) store_release(p.flags + w, 1u);
+}
+
 // Piece k (in processing order) of the work-line segment of warp `slot`:
 // warp-group w, tiles [ta, tb).  Returns false past the last piece.  The
 // order is: the head of the last warp-group (if the segment ends inside it),
@@ -69,30 +99,12 @@ __global__ void __launch_bounds__(kKsThreads, 8 / ST)
   for (uint32_t k = 0;; ++k) {
     uint32_t w, ta, tb;
     if (!segment_piece(p, NT, slot, k, w, ta, tb)) break;
-    if (ta > 0) {  // tail: wait for the head piece of this warp-group
-      uint32_t it = 0;
-      bool ok = true;
-      while (load_acquire(p.flags + w) != p.wait_epoch) {
-        if (++it > p.spin_limit) {
-          ok = false;
-          break;
-        }
-        __nanosleep(256);
-      }
-      if (!__all_sync(0xffffffffu, ok)) {
-        if (lane == 0) atomicOr(p.err, kErrTimeout);
-        continue;
-      }
-    }
+    if (ta > 0 && !await_head(p, w, lane)) continue;
     const uint32_t g = w * 32 + lane;
     if (g < a.G)
       run_piece<LAYOUT, U, ST>(a, e, g, zs + threadIdx.x, zs + 32 * kKsThreads + threadIdx.x,
                                zs + kTileBufWords + ST * threadIdx.x, ta, tb);
-    if (ta == 0 && tb < NT) {  // head: publish the state for the next segment
-      __threadfence();
-      __syncwarp();
-      if (lane == 0) store_release(p.flags + w, p.epoch);
-    }
+    if (ta == 0 && tb < NT) publish_head(p, w, lane);
   }
 }
 
@@ -225,24 +237,9 @@ __global__ void __launch_bounds__(2 * kKsThreads, 1)
     if (!segment_piece(p, NT, slot, k, w, ta, tb)) break;
     const uint32_t g = w * 32 + lane;
     if (clocker) {
-      if (ta > 0) {  // tail: wait for the head piece of this warp-group
-        uint32_t it = 0;
-        bool ok = true;
-        while (load_acquire(p.flags + w) != p.wait_epoch) {
-          if (++it > p.spin_limit) {
-            ok = false;
-            break;
-          }
-          __nanosleep(256);
-        }
-        if (!__all_sync(0xffffffffu, ok) && lane == 0) atomicOr(p.err, kErrTimeout);
-      }
+      if (ta > 0) await_head(p, w, lane);
       clock_piece<U>(a, g, zb0, zb1, par, 1 + pair, ta, tb);
-      if (ta == 0 && tb < NT) {  // head: publish the state for the next segment
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) store_release(p.flags + w, p.epoch);
-      }
+      if (ta == 0 && tb < NT) publish_head(p, w, lane);
     } else {
       emit_piece<LAYOUT, ST>(a, e, g, zb0, zb1, zs + kTileBufWords + ST * t, par, 1 + pair, ta,
                              tb);

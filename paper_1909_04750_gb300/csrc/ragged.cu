@@ -239,20 +239,7 @@ __global__ void __launch_bounds__(2 * kKsThreads, 1)
     const uint32_t w = uint32_t(a.line.order[pos]), g = w * 32 + lane;
     const uint32_t ta = kSnapTiles * uint32_t(ba), tb = kSnapTiles * uint32_t(bb);
     const bool ends = a.line.blocks[pos] + bb == a.line.blocks[pos + 1];
-    if (clocker) {
-      if (ta > 0) {  // tail: wait for the head piece of this warp-group
-        uint32_t it = 0;
-        bool ok = true;
-        while (load_acquire(p.flags + w) != p.wait_epoch) {
-          if (++it > p.spin_limit) {
-            ok = false;
-            break;
-          }
-          __nanosleep(256);
-        }
-        if (!__all_sync(0xffffffffu, ok) && lane == 0) atomicOr(p.err, kErrTimeout);
-      }
-    }
+    if (clocker && ta > 0) await_head(p, w, lane);
     // The lane table: the clock side fills what it reads itself (snap), the
     // emission side the rest.  Every thread uses its own columns only.
     uint64_t words = 0;
@@ -270,11 +257,7 @@ __global__ void __launch_bounds__(2 * kKsThreads, 1)
     }
     if (clocker) {
       ragged_clock_piece<LAYOUT>(a, lt, g, zb0, zb1, par, 1 + pair, ta, tb, ends);
-      if (!ends) {  // head: publish the state for the next segment
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) store_release(p.flags + w, p.epoch);
-      }
+      if (!ends) publish_head(p, w, lane);
     } else {
 #pragma unroll 1
       for (uint32_t T = ta; T < tb; ++T) {
