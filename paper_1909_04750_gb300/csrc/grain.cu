@@ -296,12 +296,11 @@ MICKEY_API int grain_generate(grain_streams *s, uint64_t n_bits, void *out, int 
   if (layout == MICKEY_LAYOUT_BITSLICED_U32 && (reinterpret_cast<uintptr_t>(out) & 3u))
     return grain_fail(MICKEY_E_ARG, "bitsliced output must be 4-byte aligned");
   // rows off the 16-byte grid cost the thread-per-group launch byte stores
-  // (1001 bits, 2^20 instances: 1196 us against 616), so those are packed at
+  // (1001 bits, 2^20 instances: 1196 us against 216), so those are packed at
   // any size
-  const bool rows16 =
-      ((n_bits + 7) / 8) % 16 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
   const uint32_t per_sm = layout == MICKEY_LAYOUT_BITSLICED_U32 ? kGrainPackedBitslicedPerSm
-                          : rows16 ? kGrainPackedBytesPerSm : ~0u / uint32_t(s->sm_count);
+                          : grain_rows16(n_bits, out)           ? kGrainPackedBytesPerSm
+                                                                : ~0u / uint32_t(s->sm_count);
   const KeystreamArgs ka{s->d_state, s->G, s->Gpad, s->n, n_bits, out};
   if (grain_use_packed(s, per_sm)) {
     if (launch_grain_packed(ka, layout, s->stream) != cudaSuccess)

@@ -75,7 +75,8 @@ __device__ __forceinline__ void grain_clock_piece(const KeystreamArgs &a, uint32
   }
 }
 
-// Row emission, whole tiles and rows on the 16-byte grid.  Grain's clock is a
+// Row emission, rows on the 16-byte grid (a last partial tile, whose words past
+// the call's end are zero, then fills a row's last word).  Grain's clock is a
 // ninth of MICKEY's, so here the emission warp's time per tile matters.
 //   * A tile is transposed in registers: one read of its 32 words, no second
 //     pass through shared memory.
@@ -95,7 +96,7 @@ constexpr int kRingSlots = 12;
 __device__ __forceinline__ void grain_flush(const uint32_t *rb, const KeystreamArgs &a, uint32_t g,
                                             uint32_t ba, uint32_t bb, int r0, int r1,
                                             uint32_t lane_mask) {
-  const uint64_t pitch = a.n_bits >> 3;
+  const uint64_t pitch = (a.n_bits + 7) >> 3;
   uint8_t *o = static_cast<uint8_t *>(a.out) + (32ull * g + uint32_t(r0)) * pitch + uint64_t(ba) * 4;
   if (bb - ba == 7) {
     const uint32_t *h0 = rb + (ba % kRingSlots) * kKsThreads;         // slots 0, 4 or 8 on
@@ -217,8 +218,9 @@ cudaError_t launch_grain_ws(const KeystreamArgs &a, int layout, const PersistArg
   e.lane_mask = tail ? (1u << tail) - 1u : ~0u;
   e.vec_ok = addr % 16 == 0 && a.n_bits % 4 == 0;
   e.word_ok = addr % 4 == 0 && ((a.n_bits + 7) / 8) % 4 == 0;
-  // rows on the 16-byte grid (a last block of fewer tiles goes out word by word)
-  e.stage = layout == MICKEY_LAYOUT_BYTES && addr % 16 == 0 && a.n_bits % 128 == 0;
+  // a last block of fewer tiles than eight goes out word by word.  2^20 instances
+  // x 16,380 bits: 1632 us, unstaged 8415
+  e.stage = layout == MICKEY_LAYOUT_BYTES && grain_rows16(a.n_bits, a.out);
   return layout == MICKEY_LAYOUT_BYTES ? launch_layout<kLayoutBytesLsb>(a, e, p, st)
                                        : launch_layout<MICKEY_LAYOUT_BITSLICED_U32>(a, e, p, st);
 }

@@ -143,6 +143,11 @@ cudaError_t launch_quarters(const KeystreamArgs &a, int layout, int sm_count, cu
 // bytes layout, any n_bits and alignment that grain_generate takes; loading and
 // the 160 initialisation clocks.  State: s0..s79 then b0..b79, rows of Gpad words.
 cudaError_t launch_grain_packed(const KeystreamArgs &a, int layout, cudaStream_t st);
+// Whether Grain's byte rows lie on the 16-byte grid: the paired launch stages
+// them then, whatever the last tile holds (a row is a whole number of words).
+inline bool grain_rows16(uint64_t n_bits, const void *out) {
+  return ((n_bits + 7) / 8) % 16 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+}
 // Grain with clock warps paired with emission warps (grain_ws.cu), any
 // n_bits and alignment; `p` as for the paired keystream launch.
 cudaError_t launch_grain_ws(const KeystreamArgs &a, int layout, const PersistArgs &p,
