@@ -312,6 +312,8 @@ void set_hand_off(const mickey_streams *s, PersistArgs &pa) {
 
 // One keystream launch of `bits` clocks into a device buffer.
 //   AUTO, few groups          one thread per instance, or four warps per warp-group
+//                             (calls of a few clocks go over to the latter earlier:
+//                             250,000 x 1 bit of bytes 24 against 15 us)
 //   GRID                      one thread per group, clocking and emitting
 //   PERSISTENT2, enough groups two clocking warps per SM sub-partition
 //   otherwise (AUTO, PERSISTENT) the paired kernel: clock warps beside emission
@@ -329,7 +331,8 @@ int launch_generate(mickey_streams *s, uint64_t bits, void *out, int layout) {
     const uint32_t sms = uint32_t(s->sm_count);
     const bool words = layout != MICKEY_LAYOUT_BYTES ||
                        ((bits + 7) / 8 % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 4 == 0);
-    if (s->G <= (words ? kPackedKeystreamPerSm : kPackedPerSm) * sms) {
+    const uint32_t per_sm = bits <= 8 ? kPackedShortPerSm : words ? kPackedKeystreamPerSm : kPackedPerSm;
+    if (s->G <= per_sm * sms) {
       CUDA_TRY(launch_packed_keystream(ka, layout, s->stream), "packed_keystream_kernel launch");
       return MICKEY_OK;
     }

@@ -191,9 +191,37 @@ void grain_release(grain_streams *s) {
 // every sub-partition has one (19456 groups; the initialisation: two).
 constexpr uint32_t kGrainPackedInitPerSm = 128;
 constexpr uint32_t kGrainPackedBitslicedPerSm = 54, kGrainPackedBytesPerSm = 86;
+// Short calls are moving states, which costs a thread per instance its
+// transposes, 1.6 us per 1000 groups (us; packed, thread per group):
+//   groups                       2719      4844      7813      12500     19456     32768
+//   bitsliced, 8 bits          13, 13    15, 13    21, 14    28, 15    40, 15    58, 20
+//   bitsliced, 256 bits        17, 23    21, 23    29, 24    -
+//   rows of one byte           14, 17    16, 17    21, 17    29, 18    40, 19    58, 25
+//   rows of 24 bits            13, 24    17, 24    21, 25    29, 26    40, 30    58, 50
+//   rows of one word           12, 14    16, 15    21, 16    28, 16    39, 15    57, 24
+// Longer rows off the 16-byte grid cost the thread-per-group launch byte
+// stores (1001 bits, 2^20 instances: 1196 against 216): packed at any size.
+constexpr uint32_t kGrainPackedShortRowsPerSm = 32, kGrainPackedThreeBytesPerSm = 64;
 
 bool grain_use_packed(const grain_streams *s, uint32_t per_sm) {
   return s->force < 0 && s->G <= per_sm * uint32_t(s->sm_count);
+}
+
+bool grain_generate_packed(const grain_streams *s, uint64_t n_bits, const void *out, int layout) {
+  if (layout == MICKEY_LAYOUT_BITSLICED_U32) {
+    // the two estimates behind the table's bitsliced lines:
+    //   packed 8.4 + (0.243 + 0.00076 n_bits) per_sm,  thread per group 12.6 + 0.0445 n_bits
+    const double per_sm = double(s->G) / s->sm_count;
+    return grain_use_packed(s, kGrainPackedBitslicedPerSm) &&
+           double(n_bits) * (0.0445 - 0.00076 * per_sm) >= 0.243 * per_sm - 4.2;
+  }
+  const uint64_t row = (n_bits + 7) / 8;
+  const uint32_t per_sm = grain_rows16(n_bits, out) ? kGrainPackedBytesPerSm
+                          : row == 1 || (row == 4 && reinterpret_cast<uintptr_t>(out) % 4 == 0)
+                              ? kGrainPackedShortRowsPerSm
+                          : row <= 3 ? kGrainPackedThreeBytesPerSm
+                                     : ~0u / uint32_t(s->sm_count);
+  return grain_use_packed(s, per_sm);
 }
 
 // Loading and initialisation clocks from device inputs.
@@ -295,31 +323,29 @@ MICKEY_API int grain_generate(grain_streams *s, uint64_t n_bits, void *out, int 
     return grain_fail(MICKEY_E_LAYOUT, "Grain takes the bitsliced or the bytes layout");
   if (layout == MICKEY_LAYOUT_BITSLICED_U32 && (reinterpret_cast<uintptr_t>(out) & 3u))
     return grain_fail(MICKEY_E_ARG, "bitsliced output must be 4-byte aligned");
-  // rows off the 16-byte grid cost the thread-per-group launch byte stores
-  // (1001 bits, 2^20 instances: 1196 us against 216), so those are packed at
-  // any size
-  const uint32_t per_sm = layout == MICKEY_LAYOUT_BITSLICED_U32 ? kGrainPackedBitslicedPerSm
-                          : grain_rows16(n_bits, out)           ? kGrainPackedBytesPerSm
-                                                                : ~0u / uint32_t(s->sm_count);
   const KeystreamArgs ka{s->d_state, s->G, s->Gpad, s->n, n_bits, out};
-  if (grain_use_packed(s, per_sm)) {
+  if (grain_generate_packed(s, n_bits, out, layout)) {
     if (launch_grain_packed(ka, layout, s->stream) != cudaSuccess)
       return grain_fail(MICKEY_E_CUDA, "grain keystream launch");
     s->pos += n_bits;
     return set_error(MICKEY_OK, "");
   }
   // Equal segments of the groups x tiles work line, one per clock warp, once
-  // there is a warp-group for each; with fewer, a warp-group per pair.  Forced
-  // hand-offs: one segment fewer than warp-groups, tails first.
+  // there is a warp-group for each; with fewer, a warp-group per pair.  Rows
+  // that are staged in blocks of eight tiles are cut between blocks (a block in
+  // two segments goes out word by word: 800,000 instances x 256 bits 72 us, 50 when not cut).
+  // Forced hand-offs: one segment fewer than warp-groups, tails first.
   const uint64_t W = (s->G + 31) / 32, NT = (n_bits + 31) / 32;
   const bool hand_off = s->force == 1;
   const uint64_t slots = std::min<uint64_t>(4ull * uint32_t(s->sm_count),
                                             hand_off ? std::max<uint64_t>(W - 1, 1) : W);
   PersistArgs pa{};
   pa.blocks = uint32_t((slots + 3) / 4);
-  pa.cooperative = slots < W;
   pa.W = uint32_t(W);
   pa.L = (W * NT + slots - 1) / slots;
+  if (layout == MICKEY_LAYOUT_BYTES && NT % 8 == 0 && grain_rows16(n_bits, out) && !hand_off)
+    pa.L = (pa.L + 7) / 8 * 8;
+  pa.cooperative = pa.L % NT != 0;        // else no warp-group is cut
   pa.flags = s->d_flags;
   pa.wait_flag = 1;
   pa.spin_limit = s->spin_limit;

@@ -62,7 +62,10 @@ cudaError_t launch_packed_init(const LoadArgs &a, uint32_t *state, cudaStream_t 
 // with two, 270 with three; a thread per group takes 334 ns until all 608
 // sub-partitions have a warp of 32 groups.  Rows of bytes that are not whole
 // words cost the emission warps byte stores: there the packed launch goes as
-// far as it beats a thread per group.
+// far as it beats a thread per group.  A call of up to 8 clocks mostly moves
+// states, which costs the packed launch its transposes (1 bit, bitsliced: 2719
+// groups 15 against 11 us, 7813 groups 24 against 11).
+constexpr uint32_t kPackedShortPerSm = 13;
 constexpr uint32_t kPackedKeystreamPerSm = 18;
 constexpr uint32_t kPackedPerSm = 52;
 
