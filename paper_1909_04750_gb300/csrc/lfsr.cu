@@ -545,6 +545,9 @@ void launch_crc_warp_poly(bool any, uint32_t grid, cudaStream_t st, const uint8_
     crc8_warp_kernel<POLY, false><<<grid, kCrcWarpBlock, 0, st>>>(d, n, len, poly, init, xorout,
                                                                   crc, cj, past, G);
 }
+bool crc_poly_has_kernel(uint8_t poly) {
+  return poly == 0x07 || poly == 0x1D || poly == 0x2F || poly == 0x31 || poly == 0x9B || poly == 0xD5;
+}
 template <class... A>
 void launch_crc_warp(uint8_t poly, A &&...a) {
   switch (poly) {
@@ -558,9 +561,51 @@ void launch_crc_warp(uint8_t poly, A &&...a) {
   }
 }
 
+// Which kernel takes n messages of len bytes (`vec`: len and the data are
+// multiples of 16 bytes, which the tiles need).  Measured on a GB300, us; the
+// warp kernel for P = 0x1D and, in brackets, for a polynomial without a kernel
+// of its own:
+//   n           len      32    64    96    112   128       160       192       256       384
+//   2^17        table    17    31    28    25    80        39
+//               tiles    20    28    36    41    43        50        58        73        103
+//               units    30    30    30    30    30 (40)   30 (42)   30 (41)   30 (39)   31 (41)
+//   2^19        table    30    80    87    86    273       181
+//               tiles    22    33    39    50    49        58        68        95        132
+//               units    73    74    74    73    74 (120)  74 (119)  74 (120)  77 (118)  79 (119)
+//   2^20        table    48    137   145   163   494       340
+//               tiles    31    49    63    80    90        117       135       173       248
+//               units    129   130   131   133   136 (229) 138 (228) 137 (229) 138 (222) 141 (226)
+// Off the 16-byte grid the table takes 128 for 2^20 messages of 100 bytes and
+// 256 for 140, the units 156 and 159 (223 and 228), so the line between them
+// stays at 112 bytes.  (Bitsliced by a thread per 32 messages, which the two
+// replace there: 258 for 60 bytes, 4212 for 1000, 2743 for 10,000 messages of
+// 1500.)
+enum class CrcRoute { kTable, kTiles, kUnits };
+CrcRoute crc_route(uint8_t poly, size_t n, size_t len, bool vec) {
+  if (len <= 112) {
+    // messages from which the tiles outrun the table, for 0, 16, 32, ... bytes
+    constexpr size_t kNever = ~size_t(0);
+    constexpr size_t kFrom[8] = {kNever, kNever, 280000, 640000, 114688, 400000, 180000, 230000};
+    return vec && n >= kFrom[len / 16] ? CrcRoute::kTiles : CrcRoute::kTable;
+  }
+  if (!vec) return CrcRoute::kUnits;
+  // The estimates behind the table (us).  A pass of 32 bytes per message is
+  // bound by latency up to about 2^19 messages; above 456 tiles (three of 2048
+  // messages per SM) there is more than one wave, and a last pass of 16 bytes
+  // then costs more.  The units take a time per 512 bytes or part of them that
+  // depends on the polynomial.  Over 15 sizes n up to 2^21 and 20 lengths the
+  // choice is never more than 4 % behind the faster one.
+  const double N = double(n) / (1 << 20);
+  const double pass = N < 0.89 ? 19.0 * N : (5.0 + 14.3 * N) * (len % 32 ? 1.17 : 1.0);
+  const double tiles = 14.0 + double((len + 31) / 32) * std::max(8.3, pass);
+  const double unit = crc_poly_has_kernel(poly) ? 116.0 : 214.0;
+  const double units = 15.0 + double((len / 16 + 31) / 32) * N * unit;
+  return tiles < units ? CrcRoute::kTiles : CrcRoute::kUnits;
+}
+
 // Host: x^e mod P over GF(2) (P with its x^8 term), bit k = coefficient of x^k.
-uint32_t gf2_mod(uint32_t a, uint32_t P) {
-  for (int b = 31; b >= 8; --b)
+uint32_t gf2_mod(uint32_t a, uint32_t P) {   // a of degree 14 at most, a product
+  for (int b = 14; b >= 8; --b)
     if (a >> b & 1u) a ^= P << (b - 8);
   return a;
 }
@@ -706,28 +751,17 @@ MICKEY_API int mickey_crc8(const uint8_t *data, size_t n, size_t len, uint8_t po
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const bool vec = len % 16 == 0 && reinterpret_cast<uintptr_t>(d_data) % 16 == 0;
-  // Which kernel.  Measured, 2^20 messages, P = 0x1D (us; in brackets 20,000):
-  //   length              28        60        100       140       1000
-  //   table, a thread     17 (11)   46 (11)   116 (12)  246 (14)  -
-  //   warp, units         140 (15)  141 (16)  147 (16)  150 (16)  256
-  //   length, aligned     32        64        128       160       208      1008
-  //   cp.async tiles      25 (13)   42 (20)   83 (35)   110 (41)  170 (55) 724
-  //   warp, units         120 (15)  120 (16)  125 (15)  126 (15)  127 (16) 238
-  // (bitsliced by a thread per 32 messages, which these replace: 258 for 60
-  // bytes, 4212 for 1000, 2743 for 10,000 messages of 1500.)  The warp kernel
-  // spends about 110 on every 512-byte chunk, or part of one, of 2^20 messages;
-  // the tiles need enough messages to fill the chip.
   const bool whole = vec && len % 512 == 0;
-  const bool tiles = vec && len > 32 && len <= 160 && n >= (size_t(1) << 19);
-  if (whole || (len > 112 && !tiles)) {
+  const CrcRoute route = whole ? CrcRoute::kUnits : crc_route(poly, n, len, vec);
+  if (route == CrcRoute::kUnits) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crc8_warp_kernel<0, false>,
                                                   kCrcWarpBlock, 0);
     const size_t G = (n + 31) / 32;
     const size_t blocks = (G + kCrcWarpBlock / 32 - 1) / (kCrcWarpBlock / 32);
     const uint32_t grid = uint32_t(std::min<size_t>(blocks, size_t(sms) * std::max(per_sm, 1)));
     launch_crc_warp(poly, !whole, grid, st, d_data, n, len, poly, init, xorout, d_crc,
-                    crc_join_matrices(poly), crc_past(poly, len), G);
-  } else if (tiles) {
+                    crc_join_matrices(poly), whole ? CrcPast{} : crc_past(poly, len), G);
+  } else if (route == CrcRoute::kTiles) {
     if (cudaFuncSetAttribute(crc8_async_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              int(kCrcTileBytes)) != cudaSuccess)
       return set_error(MICKEY_E_CUDA, "crc kernel shared memory");
