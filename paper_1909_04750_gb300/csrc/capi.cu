@@ -357,8 +357,8 @@ int launch_generate(mickey_streams *s, uint64_t bits, void *out, int layout) {
   if (use_persistent(s, mode)) {
     const uint64_t slots = uint64_t(s->persist_blocks) * per_sm * 4;
     pa.blocks = uint32_t(s->persist_blocks) * per_sm;
-    pa.cooperative = 1;
     pa.L = (W * NT + slots - 1) / slots;
+    pa.cooperative = pa.L % NT != 0;     // else no warp-group is cut
   } else {  // one warp-group per clock/emission pair, four pairs per block
     pa.blocks = uint32_t((W + 3) / 4);
     pa.cooperative = 0;

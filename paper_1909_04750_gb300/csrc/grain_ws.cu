@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(2 * kKsThreads, 1)
     if (threadIdx.x < kKsThreads) {
       if (ta > 0) await_head(p, w, lane);
       grain_clock_piece<LAYOUT>(a, g, zb0, zb1, par, 1 + pair, ta, tb);
+      if (ta > 0) take_back(p, w, lane);
       if (ta == 0 && tb < NT) publish_head(p, w, lane);
     } else if (LAYOUT == kLayoutBytesLsb && e.stage) {
       grain_emit_rows(a, g, zb0, zb1, zs + kTileBufWords + t, par, 1 + pair, ta, tb,

@@ -18,11 +18,7 @@ __device__ __forceinline__ void store_release(uint32_t *p, uint32_t v) {
 }
 
 // The bounded wait of a tail piece (the whole warp) for the head of its
-// warp-group.  The flag is taken back at once, so the flags are zero again when
-// the launch ends: nothing clears them between calls, and a captured call can
-// be replayed.  When the wait runs out the error flag is raised, and the flag,
-// which the head may still set, stays; the call that reports the error clears
-// them all.
+// warp-group; when it runs out the error flag is raised.
 __device__ __forceinline__ bool await_head(const PersistArgs &p, uint32_t w, uint32_t lane) {
   uint32_t it = 0;
   bool ok = true;
@@ -34,11 +30,16 @@ __device__ __forceinline__ bool await_head(const PersistArgs &p, uint32_t w, uin
     __nanosleep(256);
   }
   ok = __all_sync(0xffffffffu, ok);
-  if (lane == 0) {
-    if (ok) *reinterpret_cast<volatile uint32_t *>(p.flags + w) = 0u;
-    else atomicOr(p.err, kErrTimeout);
-  }
+  if (!ok && lane == 0) atomicOr(p.err, kErrTimeout);
   return ok;
+}
+// After the tail piece the flag is taken back, so that all are zero again when
+// the launch ends: nothing clears them between calls, and a captured call can
+// be replayed.  (Right after the wait it cost 1 us per piece: the compiler then
+// kept the address through the piece.)  Only a head whose tail gave up may
+// leave one set; the call that reports the error clears them.
+__device__ __forceinline__ void take_back(const PersistArgs &p, uint32_t w, uint32_t lane) {
+  if (lane == 0) *reinterpret_cast<volatile uint32_t *>(p.flags + w) = 0u;
 }
 // The end of a head piece: the warp's stores of the state, then the flag.
 __device__ __forceinline__ void publish_head(const PersistArgs &p, uint32_t w, uint32_t lane) {
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(kKsThreads, 8 / ST)
     if (g < a.G)
       run_piece<LAYOUT, U, ST>(a, e, g, zs + threadIdx.x, zs + 32 * kKsThreads + threadIdx.x,
                                zs + kTileBufWords + ST * threadIdx.x, ta, tb);
+    if (ta > 0) take_back(p, w, lane);
     if (ta == 0 && tb < NT) publish_head(p, w, lane);
   }
 }
@@ -239,6 +241,7 @@ __global__ void __launch_bounds__(2 * kKsThreads, 1)
     if (clocker) {
       if (ta > 0) await_head(p, w, lane);
       clock_piece<U>(a, g, zb0, zb1, par, 1 + pair, ta, tb);
+      if (ta > 0) take_back(p, w, lane);
       if (ta == 0 && tb < NT) publish_head(p, w, lane);
     } else {
       emit_piece<LAYOUT, ST>(a, e, g, zb0, zb1, zs + kTileBufWords + ST * t, par, 1 + pair, ta,
@@ -277,7 +280,7 @@ cudaError_t launch_persistent_kernel(const KeystreamArgs &a, const EmitCtx &e,
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
+  attr[0].val.cooperative = p.cooperative ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, keystream_persistent_kernel<LAYOUT, U, ST>, a, e, p);

@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(2 * kKsThreads, 1)
     }
     if (clocker) {
       ragged_clock_piece<LAYOUT>(a, lt, g, zb0, zb1, par, 1 + pair, ta, tb, ends);
+      if (ta > 0) take_back(p, w, lane);
       if (!ends) publish_head(p, w, lane);
     } else {
 #pragma unroll 1
