@@ -140,6 +140,30 @@ __global__ void __launch_bounds__(kInitT) grain_init_kernel(GrainInitArgs a) {
   }
 }
 
+// A few clocks of the bitsliced layout, a thread per group: no more than moving
+// the states.  The paired launch clocks a whole tile for them, and with more
+// warp-groups than clock warps one behind the other.
+__global__ void __launch_bounds__(kInitT) grain_short_kernel(KeystreamArgs a, uint32_t lane_mask) {
+  const uint32_t g = blockIdx.x * kInitT + threadIdx.x;
+  if (g >= a.G) return;
+  if (g != a.G - 1) lane_mask = ~0u;
+  const size_t P = a.Gpad;
+  uint32_t s[kG], b[kG];
+#pragma unroll
+  for (int i = 0; i < kG; ++i) {
+    s[i] = a.state[size_t(i) * P + g];
+    b[i] = a.state[size_t(kG + i) * P + g];
+  }
+  uint32_t *o = static_cast<uint32_t *>(a.out) + size_t(g) * a.n_bits;
+#pragma unroll 1
+  for (uint32_t c = 0; c < a.n_bits; ++c) o[c] = grain_clock_shift(s, b) & lane_mask;
+#pragma unroll
+  for (int i = 0; i < kG; ++i) {
+    a.state[size_t(i) * P + g] = s[i];
+    a.state[size_t(kG + i) * P + g] = b[i];
+  }
+}
+
 // Logic ops per clock per 32-lane group, as written above (keystream clock
 // including z, or an initialisation clock).
 constexpr int kGrainOps = 10 + 3 + 23;
@@ -201,6 +225,10 @@ constexpr uint32_t kGrainPackedBitslicedPerSm = 54, kGrainPackedBytesPerSm = 86;
 //   rows of one word           12, 14    16, 15    21, 16    28, 16    39, 15    57, 24
 // Longer rows off the 16-byte grid cost the thread-per-group launch byte
 // stores (1001 bits, 2^20 instances: 1196 against 216): packed at any size.
+// Bitsliced calls of up to this many clocks that are not packed take
+// grain_short_kernel (us; paired launch, this kernel: 500,000 instances x 8 bits
+// 14.6, 11.5; x 16 15.3, 13.2; 2^21 x 8 32.3, 20.2; x 16 34.4, 24.7).
+constexpr uint64_t kGrainShortBits = 16;
 constexpr uint32_t kGrainPackedShortRowsPerSm = 32, kGrainPackedThreeBytesPerSm = 64;
 
 bool grain_use_packed(const grain_streams *s, uint32_t per_sm) {
@@ -326,6 +354,15 @@ MICKEY_API int grain_generate(grain_streams *s, uint64_t n_bits, void *out, int 
   const KeystreamArgs ka{s->d_state, s->G, s->Gpad, s->n, n_bits, out};
   if (grain_generate_packed(s, n_bits, out, layout)) {
     if (launch_grain_packed(ka, layout, s->stream) != cudaSuccess)
+      return grain_fail(MICKEY_E_CUDA, "grain keystream launch");
+    s->pos += n_bits;
+    return set_error(MICKEY_OK, "");
+  }
+  if (layout == MICKEY_LAYOUT_BITSLICED_U32 && n_bits <= kGrainShortBits && s->force < 0) {
+    const uint32_t tail = uint32_t(s->n & 31u);
+    grain_short_kernel<<<(s->G + kInitT - 1) / kInitT, kInitT, 0, s->stream>>>(
+        ka, tail ? (1u << tail) - 1u : ~0u);
+    if (cudaGetLastError() != cudaSuccess)
       return grain_fail(MICKEY_E_CUDA, "grain keystream launch");
     s->pos += n_bits;
     return set_error(MICKEY_OK, "");

@@ -196,8 +196,8 @@ __device__ __forceinline__ void grain_body(uint32_t (&s)[kG], uint32_t (&b)[kG],
   });
 }
 
-// One clock with the registers physically shifted (rotation stays 0): the
-// tail of a call, fewer than 80 clocks.
+// One clock with the registers physically shifted (rotation stays 0), for a
+// few clocks.
 __device__ __forceinline__ uint32_t grain_clock_shift(uint32_t (&s)[kG], uint32_t (&b)[kG]) {
   const uint32_t s0 = s[0], b0 = b[0];
   const uint32_t z = grain_clock<0, false>(s, b);   // writes the new bits to slot 0

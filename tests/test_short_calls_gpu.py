@@ -129,3 +129,25 @@ def test_grain_one_byte_costs_about_what_its_bits_cost():
             best = min(best, 1e3 * e0.elapsed_time(e1))
         us[layout] = best
     assert us["bytes"] < 2 * us["bitsliced"], us
+
+
+# above the packed launch's line: up to 16 clocks in a kernel of their own, the
+# paired launch from 17; the lanes past the last instance stay zero
+@pytest.mark.parametrize("n", [60 * 152 * 32 + 11, 700_003])
+def test_grain_few_bitsliced_clocks(n):
+    from oracle import grain as og
+    from paper_1909_04750_gb300.grain import GrainStreams
+    s = workloads.grain_streams(n, seed=43)
+    idx = _sample(n)
+    st = GrainStreams(torch.from_numpy(s.keys).cuda(), torch.from_numpy(s.ivs).cuda())
+    calls = [16, 1, 17, 15, 2, 32, 7]
+    bits = np.unpackbits(og.batch_bytes(s.keys[idx], s.ivs[idx], sum(calls), threads=THREADS), axis=1,
+                         bitorder="little")
+    at = 0
+    for b in calls:
+        words = st.generate(b, "bitsliced").view((n + 31) // 32, b).cpu().numpy().view(np.uint32)
+        got = (words[idx // 32] >> (idx % 32).astype(np.uint32)[:, None]) & 1
+        assert np.array_equal(got, bits[:, at:at + b])
+        assert not (words[-1] >> np.uint32(n % 32)).any()
+        at += b
+    st.sync()
