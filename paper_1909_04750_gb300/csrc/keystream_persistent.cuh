@@ -233,20 +233,33 @@ __global__ void __launch_bounds__(2 * kKsThreads, 1)
   const uint64_t NT = (a.n_bits + 31) >> 5;
   uint32_t *zb0 = zs + t, *zb1 = zs + 32 * kKsThreads + t;
   uint32_t par = 0;
-#pragma unroll 1
-  for (uint32_t k = 0;; ++k) {
+  auto clock_side = [&](uint32_t w, uint32_t ta, uint32_t tb) {
+    if (ta > 0) await_head(p, w, lane);
+    clock_piece<U>(a, w * 32 + lane, zb0, zb1, par, 1 + pair, ta, tb);
+    if (ta > 0) take_back(p, w, lane);
+    if (ta == 0 && tb < NT) publish_head(p, w, lane);
+  };
+  auto emit_side = [&](uint32_t w, uint32_t ta, uint32_t tb) {
+    emit_piece<LAYOUT, ST>(a, e, w * 32 + lane, zb0, zb1, zs + kTileBufWords + ST * t, par, 1 + pair,
+                           ta, tb);
+  };
+  auto pieces = [&](auto &&side) {
     uint32_t w, ta, tb;
-    if (!segment_piece(p, NT, slot, k, w, ta, tb)) break;
-    const uint32_t g = w * 32 + lane;
-    if (clocker) {
-      if (ta > 0) await_head(p, w, lane);
-      clock_piece<U>(a, g, zb0, zb1, par, 1 + pair, ta, tb);
-      if (ta > 0) take_back(p, w, lane);
-      if (ta == 0 && tb < NT) publish_head(p, w, lane);
-    } else {
-      emit_piece<LAYOUT, ST>(a, e, g, zb0, zb1, zs + kTileBufWords + ST * t, par, 1 + pair, ta,
-                             tb);
-    }
+#pragma unroll 1
+    for (uint32_t k = 0; segment_piece(p, NT, slot, k, w, ta, tb); ++k) side(w, ta, tb);
+  };
+  // A loop of its own for each side spills less: 2^21 x 256 bits of u32 352 ->
+  // 338 us.  The bitsliced emission, which is short, does as well in one loop,
+  // and calls of a few clocks better (2^21 x 1 bit 27.7 against 30.8).
+  if constexpr (LAYOUT == MICKEY_LAYOUT_BITSLICED_U32) {
+    pieces([&](uint32_t w, uint32_t ta, uint32_t tb) {
+      if (clocker) clock_side(w, ta, tb);
+      else emit_side(w, ta, tb);
+    });
+  } else if (clocker) {
+    pieces(clock_side);
+  } else {
+    pieces(emit_side);
   }
 }
 
