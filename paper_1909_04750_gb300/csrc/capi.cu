@@ -390,6 +390,22 @@ uint64_t ragged_packed(size_t n, const uint64_t *n_bits, int layout, uint64_t *o
   return off;
 }
 
+// Copy m lengths and return the longest, in one pass (a pass of its own over
+// 2^20 lengths cost the call 0.7 ms): four maxima, so that they do not wait for
+// one another.
+uint64_t copy_longest(const uint64_t *src, size_t m, uint64_t *dst) {
+  uint64_t top[4] = {0, 0, 0, 0};
+  size_t i = 0;
+  for (; i + 4 <= m; i += 4)
+    for (int k = 0; k < 4; ++k) {
+      const uint64_t v = src[i + k];
+      dst[i + k] = v;
+      top[k] = v > top[k] ? v : top[k];
+    }
+  for (; i < m; ++i) top[0] = std::max(top[0], dst[i] = src[i]);
+  return std::max(std::max(top[0], top[1]), std::max(top[2], top[3]));
+}
+
 // True when every stream asks for the same number of bits and the offsets
 // (NULL = packed) are the packed ones: row i at i * row bytes, group g's
 // words at g * 4 * n_bits.
@@ -562,7 +578,6 @@ int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
   const int kb = s->ragged_flip;
   CUDA_TRY(cudaEventSynchronize(s->ev_h2d[kb]), "staging buffer");  // its last copy is done
   uint64_t *h = s->h_ragged[kb];
-  std::copy(n_bits, n_bits + n, h);
   if (out_offsets)
     std::copy(out_offsets, out_offsets + n_off, h + n);
   else
@@ -571,13 +586,13 @@ int mickey_generate_ragged(mickey_streams *s, const uint64_t *n_bits, void *out,
   const bool packed = (c.set ? c.mode : s->mode) == MICKEY_MODE_AUTO && use_packed(s);
   const uint64_t slots = std::min<uint64_t>(W, 4ull * uint32_t(s->persist_blocks));
   RaggedLine line{};
-  if (!packed) {
-    std::vector<uint64_t> blocks(W, 0);
-    for (size_t w = 0; w < W; ++w) {
-      for (size_t i = 1024 * w; i < std::min(n, 1024 * w + 1024); ++i)
-        blocks[w] = std::max(blocks[w], n_bits[i]);
-      blocks[w] = (blocks[w] + kRaggedBlockBits - 1) / kRaggedBlockBits;
-    }
+  if (packed) {
+    std::copy(n_bits, n_bits + n, h);
+  } else {
+    std::vector<uint64_t> blocks(W);
+    for (size_t w = 0; w < W; ++w)
+      blocks[w] = (copy_longest(n_bits + 1024 * w, std::min<size_t>(n - 1024 * w, 1024),
+                                h + 1024 * w) + kRaggedBlockBits - 1) / kRaggedBlockBits;
     uint64_t *order = h + n + n_off;
     line = ragged_cuts(blocks.data(), uint32_t(W), slots, order, order + W);
     line.order = s->d_ragged + n + n_off;    // where the copy below puts them
