@@ -309,7 +309,8 @@ MICKEY_API int mickey_batch_run(mickey_batch *b, const void *keys, const void *i
  * warp, a stream per lane (about ten times less time per clock than a thread
  * per group, for long streams whose sequential clocks bound the run); 0
  * disables the split path.  A new plan of up to 400 groups per SM splits
- * every group (split_clocks 1), a larger one none.  Re-captures the graph. */
+ * every group (split_clocks 1) unless their lengths are alike and just fill the
+ * chip's warps, a larger one none.  Re-captures the graph. */
 MICKEY_API int mickey_batch_set_config(mickey_batch *b, int unroll, int blocks_per_sm,
                                        uint64_t split_clocks);
 /* Where the split groups run (re-captures the graph):

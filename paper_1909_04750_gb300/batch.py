@@ -125,11 +125,13 @@ def tune(batch: Batch, keys, ivs, out: torch.Tensor, refresh: bool = False) -> d
     # issue slots with the critical group's warp) are searched together
     mx = batch.max_clocks
     for b in (1, 2):
-        # no split path at all only where the longest group is short
-        for sc in ((0,) if mx <= 1 << 16 else ()) + (mx // 4, mx // 8, mx // 16, mx // 32,
+        # no split path at all only where the longest group is short or the
+        # lengths are alike
+        alike = 2 * batch.total_clocks >= mx * ((batch.n + 31) // 32)
+        for sc in ((0,) if mx <= 1 << 16 or alike else ()) + (mx // 4, mx // 8, mx // 16, mx // 32,
                                                      mx // 64):
             trial(4, b, sc)
-    trial(4, 1, 1)      # every group split, as a new plan of up to 400 groups per SM has it
+    trial(4, 1, 1)      # every group split, as most new plans of up to 400 groups per SM
     best = min(cands, key=lambda c: c["ms"])
     trial(2, best["blocks_per_sm"], best["split_clocks"])
     best = min(cands, key=lambda c: c["ms"])

@@ -297,31 +297,43 @@ void batch_release(mickey_batch *b) {
 // Time per clock (ns) of a split warp when 1, 2, 3 or 4 share an SM
 // sub-partition (row stores included).
 constexpr double kPackedNs[4] = {29.0, 52.0, 76.0, 100.0};
-// Up to this many groups per SM a new plan splits every group.  A thread item
-// clocks 32 groups at 820 ns per clock (1140 when two share a sub-partition),
-// so it wins only once there are items for every warp and their lengths are
-// alike.  Measured, all split against the best of no split (ms): 20,000
-// streams of 2^10..2^18 bits 7.0, 158; 100,000 of 2^10..2^22 109, 2860;
-// 700,000 of 2^13 7.57, 9.99; 1.5 M of 2^12 8.32, 8.95; 4 M of 2^10..2^13
-// 18.5, 17.9 (the last three with a packed clock 10 % slower than now).
+// Time per clock (ns) of the thread items: kThreadNs for a lone one on a
+// sub-partition, kThreadMoreNs on top when all the resident warps have one (row
+// stores of all of them at a time).
+constexpr double kThreadNs = 850.0, kThreadMoreNs = 690.0;
+// A new plan splits every group where that is estimated to take less time than
+// thread items, up to this many groups per SM.  Thread items (32 groups) win
+// only where there is one for nearly every resident warp and their lengths are
+// alike.  Measured (152 SMs, ms; all split, the best of no split):
+//   items (1024 streams)    304         608         1064        1216        1400        1824
+//   2^13 bits each          3.41, 6.69  6.76, 7.17  11.4, 12.0  13.2, 12.8  15.1, 17.5  19.7, 19.7
+//   2^12 .. 2^13            2.69, 6.59  4.98, 6.71  8.66, 9.93  9.85, 10.6  11.5, 13.3  14.8, 15.8
+//   2^10 .. 2^13, log       1.60, 6.14  2.93, 6.32  5.04, 6.86  5.71, 6.94  6.69, 7.20  8.56, 9.47
+//   2^10 .. 2^16, log       6.31, 46.9  12.2, 48.2  21.2, 50.5  24.2, 50.8  28.0, 51.2  36.4, 52.8
 constexpr uint32_t kSplitAllPerSm = 400;
 
-// The arrangement of a new plan: all groups split, with as many warps per SM
-// sub-partition as finish first (few while the longest group's chain is what
+// The arrangement of a new plan, and with all groups split as many warps per
+// SM sub-partition as finish first (few while the longest group's chain is what
 // takes the time, more when the groups have to share the chip anyway).
 void plan_split(mickey_batch *b) {
-  if (b->G <= kSplitAllPerSm * uint32_t(b->sm_count)) {
-    b->split_clocks = 1;
-    b->n_split = b->G;
-  }
-  double best = 1e300;
+  double split = 1e300;
   for (int k = 0; k < 4; ++k) {
     const double t = std::max(double(b->max_clocks) * kPackedNs[k],
                               double(b->total_clocks) * kPackedNs[k] / ((k + 1) * 4.0 * b->sm_count));
-    if (t < best) {
-      best = t;
+    if (t < split) {
+      split = t;
       b->split_warps = k + 1;
     }
+  }
+  // thread items in waves of the resident warps, each as long as its first, the longest
+  const size_t R = size_t(b->sm_count) * b->blocks_per_sm * 4, items = (size_t(b->G) + 31) / 32;
+  double threads = 0.0;
+  for (size_t i = 0; i < items; i += R)
+    threads += double(b->group_clocks[32 * i]) *
+               (kThreadNs + kThreadMoreNs * double(std::min(R, items - i)) / double(R));
+  if (b->G <= kSplitAllPerSm * uint32_t(b->sm_count) && split <= threads) {
+    b->split_clocks = 1;
+    b->n_split = b->G;
   }
 }
 
