@@ -305,8 +305,8 @@ MICKEY_API int mickey_batch_run(mickey_batch *b, const void *keys, const void *i
                                 int mem);
 /* Launch configuration of the batch's keystream kernel: clocks per inner
  * step (2 or 4), resident blocks of 4 warps per SM (1 or 2), and
- * split_clocks: groups needing more clocks than this are each run by a whole
- * warp, a stream per lane (about ten times less time per clock than a thread
+ * split_clocks: groups needing more clocks than this (1: all groups) are each
+ * run by a whole warp, a stream per lane (about ten times less time per clock than a thread
  * per group, for long streams whose sequential clocks bound the run); 0
  * disables the split path.  A new plan of up to 400 groups per SM splits
  * every group (split_clocks 1) unless their lengths are alike and just fill the

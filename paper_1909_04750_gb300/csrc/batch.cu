@@ -530,8 +530,8 @@ MICKEY_API int mickey_batch_set_config(mickey_batch *b, int unroll, int blocks_p
   b->unroll = unroll;
   b->blocks_per_sm = blocks_per_sm;
   b->split_clocks = split_clocks;
-  uint32_t ns = 0;
-  if (split_clocks)
+  uint32_t ns = split_clocks == 1 ? b->G : 0;   // 1: every group, those of 0 or 1 clocks too
+  if (split_clocks > 1)
     while (ns < b->G && b->group_clocks[ns] > split_clocks) ++ns;
   b->n_split = ns;
   return capture(b) == cudaSuccess ? MICKEY_OK : MICKEY_E_CUDA;

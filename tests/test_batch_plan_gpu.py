@@ -60,3 +60,20 @@ def test_batch_above_the_packed_loading_sampled(split):
     for k, i in enumerate(idx):
         o, c = int(b.offsets[i]), (int(nb[i]) + 7) // 8
         assert np.array_equal(host[o:o + c], np.asarray(want[k])[:c]), i
+
+
+def test_a_reported_configuration_can_be_set_again():
+    # 40 of 80 streams empty: a whole group has nothing to clock
+    from paper_1909_04750_gb300.batch import Batch
+    s = workloads.plain_scale(80)
+    nb = np.where(np.arange(80) % 2, 4096, 0).astype(np.uint64)
+    b = Batch(nb, s.iv_lens)
+    cfg = b.get_config()
+    assert cfg["split_groups"] == 3
+    b.set_config(cfg["unroll"], cfg["blocks_per_sm"], cfg["split_clocks"], cfg["split_mode"])
+    assert b.get_config() == cfg
+    out = b.run(torch.from_numpy(s.keys).cuda(), torch.from_numpy(s.ivs).cuda())
+    b.sync()
+    want = oracle.batch_bytes(s.keys, s.ivs, s.iv_lens, nb, threads=THREADS)
+    for got, row in zip(b.rows(out), want):
+        assert np.array_equal(got, np.asarray(row)[:got.size])
