@@ -164,7 +164,8 @@ __device__ __forceinline__ void batch_group(const BatchArgs &a, uint8_t *out, ui
 
 // Store word w (memory byte order) of tile t of a row at o with `bits`
 // keystream bits (split path: row address and length held in registers).
-__device__ __forceinline__ void store_row(uint8_t *o, uint64_t bits, uint32_t t, uint32_t w) {
+template <class T>
+__device__ __forceinline__ void store_row(uint8_t *o, uint64_t bits, T t, uint32_t w) {
   const uint64_t b0 = uint64_t(t) << 5;
   if (b0 >= bits) return;
   o += b0 >> 3;
@@ -179,16 +180,18 @@ __device__ __forceinline__ void store_row(uint8_t *o, uint64_t bits, uint32_t t,
 }
 
 // One warp per group (split path), a stream per lane (packed.cuh): the group
-// runs as long as its longest lane.
+// runs as long as its longest lane.  T counts tiles: 64 bits only for batches
+// with a stream of 2^37 bits or more (the loop takes 2.6 % longer with them).
+template <class T>
 __device__ __forceinline__ void packed_group(const uint32_t *state, size_t P, uint32_t g,
                                              uint64_t clocks, uint8_t *row, uint64_t bits,
                                              uint32_t lane) {
   Packed q;
   packed_load(q, state, P, g, lane);
-  const uint32_t full = uint32_t(clocks >> 5), whole = uint32_t(bits >> 5);
+  const T full = T(clocks >> 5), whole = T(bits >> 5);
   uint32_t *o = reinterpret_cast<uint32_t *>(row);
 #pragma unroll 1
-  for (uint32_t t = 0; t < full; ++t) {
+  for (T t = 0; t < full; ++t) {
     const uint32_t w = __byte_perm(packed_clocks<32>(q), 0u, 0x0123);
     if (t < whole) o[t] = w;
     else store_row(row, bits, t, w);       // the lane ends in this tile, or has
@@ -199,14 +202,16 @@ __device__ __forceinline__ void packed_group(const uint32_t *state, size_t P, ui
 
 // In the persistent kernel as a function of its own, with a register
 // allocation of its own instead of the one-thread-per-group path's 255.
+template <class T>
 __device__ __noinline__ void packed_group_call(const uint32_t *state, size_t P, uint32_t g,
                                                uint64_t clocks, uint8_t *row, uint64_t bits,
                                                uint32_t lane) {
-  packed_group(state, P, g, clocks, row, bits, lane);
+  packed_group<T>(state, P, g, clocks, row, bits, lane);
 }
 
 // Split kernel: one-warp blocks take the split groups (0 .. n_split-1,
 // longest first) one at a time.
+template <class T>
 __global__ void __launch_bounds__(32) batch_split_kernel(BatchArgs a) {
   const uint32_t lane = threadIdx.x;
   uint8_t *out = a.params->out;
@@ -217,15 +222,15 @@ __global__ void __launch_bounds__(32) batch_split_kernel(BatchArgs a) {
     item = __shfl_sync(0xffffffffu, item, 0);
     if (item >= a.n_split) break;
     const uint64_t slot = uint64_t(item) * 32 + lane;
-    packed_group(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
-                 a.slot_bits[slot], lane);
+    packed_group<T>(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
+                    a.slot_bits[slot], lane);
   }
 }
 
 // Persistent kernel: its first split_items items are split groups, run by
 // a whole warp each; then items of 32 consecutive groups from group n_split
 // on, one group per thread.
-template <int U>
+template <int U, class T>
 __global__ void __launch_bounds__(kBatchThreads) batch_kernel(BatchArgs a) {
   __shared__ uint32_t zs[2 * 32 * kBatchThreads];
   const uint32_t lane = threadIdx.x & 31u;
@@ -238,8 +243,8 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(BatchArgs a) {
     if (item >= a.n_items) break;
     if (item < a.split_items) {
       const uint64_t slot = uint64_t(item) * 32 + lane;
-      packed_group_call(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
-                   a.slot_bits[slot], lane);
+      packed_group_call<T>(a.state, a.Gpad, item, a.group_bits[item], out + a.slot_off[slot],
+                           a.slot_bits[slot], lane);
       continue;
     }
     const uint32_t g = a.n_split + (item - a.split_items) * 32 + lane;
@@ -312,6 +317,19 @@ constexpr double kThreadNs = 850.0, kThreadMoreNs = 690.0;
 //   2^10 .. 2^16, log       6.31, 46.9  12.2, 48.2  21.2, 50.5  24.2, 50.8  28.0, 51.2  36.4, 52.8
 constexpr uint32_t kSplitAllPerSm = 400;
 
+// Clocks from which a group's tiles need a 64-bit count.
+constexpr uint64_t kThreadClocks = 1ull << 37;
+
+// The groups that split_clocks splits (1: every group, those of 0 or 1 clocks
+// too), and in any case those too long for the thread items' 32-bit count.
+void count_split(mickey_batch *b) {
+  const uint64_t most = b->split_clocks ? std::min(b->split_clocks, kThreadClocks - 1)
+                                        : kThreadClocks - 1;
+  uint32_t ns = b->split_clocks == 1 ? b->G : 0;
+  while (ns < b->G && b->group_clocks[ns] > most) ++ns;
+  b->n_split = ns;
+}
+
 // The arrangement of a new plan, and with all groups split as many warps per
 // SM sub-partition as finish first (few while the longest group's chain is what
 // takes the time, more when the groups have to share the chip anyway).
@@ -331,10 +349,8 @@ void plan_split(mickey_batch *b) {
   for (size_t i = 0; i < items; i += R)
     threads += double(b->group_clocks[32 * i]) *
                (kThreadNs + kThreadMoreNs * double(std::min(R, items - i)) / double(R));
-  if (b->G <= kSplitAllPerSm * uint32_t(b->sm_count) && split <= threads) {
-    b->split_clocks = 1;
-    b->n_split = b->G;
-  }
+  if (b->G <= kSplitAllPerSm * uint32_t(b->sm_count) && split <= threads) b->split_clocks = 1;
+  count_split(b);
 }
 
 // Capture load + preclock, then the split kernel and the thread kernel as
@@ -366,20 +382,26 @@ cudaError_t capture(mickey_batch *b) {
     BatchArgs ba{b->d_state, b->G, b->Gpad, b->d_slot, b->d_slot + 32 * size_t(b->Gpad),
                  b->d_slot + 64 * size_t(b->Gpad), b->n_split, split_items,
                  split_items + (b->G - b->n_split + 31) / 32, b->d_queue, b->d_params};
+    const bool wide = b->max_clocks >= kThreadClocks;
     if (own) {   // the split groups on a branch of their own
       cudaEventRecord(fork, cs);
       cudaStreamWaitEvent(cs2, fork, 0);
       const uint32_t per = b->n_split == b->G ? uint32_t(b->split_warps) : 1u;
       const uint32_t warps = std::min<uint32_t>(b->n_split, uint32_t(b->sm_count) * 4u * per);
-      batch_split_kernel<<<warps, 32, 0, cs2>>>(ba);
+      if (wide)
+        batch_split_kernel<uint64_t><<<warps, 32, 0, cs2>>>(ba);
+      else
+        batch_split_kernel<uint32_t><<<warps, 32, 0, cs2>>>(ba);
       cudaEventRecord(join, cs2);
     }
     if (ba.n_items) {
       const uint32_t grid = uint32_t(b->sm_count * b->blocks_per_sm);
-      if (b->unroll == 2)
-        batch_kernel<2><<<grid, kBatchThreads, 0, cs>>>(ba);
+      if (wide)
+        batch_kernel<4, uint64_t><<<grid, kBatchThreads, 0, cs>>>(ba);
+      else if (b->unroll == 2)
+        batch_kernel<2, uint32_t><<<grid, kBatchThreads, 0, cs>>>(ba);
       else
-        batch_kernel<4><<<grid, kBatchThreads, 0, cs>>>(ba);
+        batch_kernel<4, uint32_t><<<grid, kBatchThreads, 0, cs>>>(ba);
     }
     if (own) cudaStreamWaitEvent(cs, join, 0);
     e = cudaStreamEndCapture(cs, &b->graph);
@@ -530,10 +552,7 @@ MICKEY_API int mickey_batch_set_config(mickey_batch *b, int unroll, int blocks_p
   b->unroll = unroll;
   b->blocks_per_sm = blocks_per_sm;
   b->split_clocks = split_clocks;
-  uint32_t ns = split_clocks == 1 ? b->G : 0;   // 1: every group, those of 0 or 1 clocks too
-  if (split_clocks > 1)
-    while (ns < b->G && b->group_clocks[ns] > split_clocks) ++ns;
-  b->n_split = ns;
+  count_split(b);
   return capture(b) == cudaSuccess ? MICKEY_OK : MICKEY_E_CUDA;
 }
 

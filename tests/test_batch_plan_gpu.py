@@ -77,3 +77,18 @@ def test_a_reported_configuration_can_be_set_again():
     want = oracle.batch_bytes(s.keys, s.ivs, s.iv_lens, nb, threads=THREADS)
     for got, row in zip(b.rows(out), want):
         assert np.array_equal(got, np.asarray(row)[:got.size])
+
+
+def test_streams_past_the_thread_items_tile_count():
+    # 2^37 bits are 2^32 tiles; planned only, such a stream runs for an hour
+    from paper_1909_04750_gb300.batch import Batch
+    nb = np.full(2000, 100, np.uint64)
+    nb[7] = 1 << 37
+    b = Batch(nb)
+    for cfg, split in (((4, 2, 0), 1), ((4, 2, 1 << 39), 1), ((4, 1, 64), 63), ((4, 1, 1), 63)):
+        b.set_config(*cfg)
+        assert b.get_config()["split_groups"] == split
+    nb[7] -= 1
+    b = Batch(nb)
+    b.set_config(4, 2, 0)
+    assert b.get_config()["split_groups"] == 0
