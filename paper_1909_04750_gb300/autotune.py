@@ -8,8 +8,8 @@ or 32-byte row chunks) -- on the handle's own streams (state saved and
 restored) and keeps the fastest; among candidates within 1 % of it the
 deepest row staging wins (whole 32-byte sectors: the least DRAM traffic at
 the same speed).  The
-choice is cached in a JSON file next to the built library so later handles
-of the same shape reuse it without timing.
+choice is cached in a JSON file next to the built library, for the library's
+present sources, so later handles of the same shape reuse it without timing.
 """
 from __future__ import annotations
 
@@ -19,6 +19,7 @@ import os
 import threading
 
 from . import _native as N
+from . import build
 
 CACHE_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build",
                           "tune_cache.json")
@@ -28,9 +29,11 @@ _lock = threading.Lock()
 
 
 def _device_key() -> str:
+    """The GPU and the library's sources: what a candidate is, and which are
+    tried, changes with them."""
     import torch
     p = torch.cuda.get_device_properties(torch.cuda.current_device())
-    return "%s|sm%d" % (p.name, p.multi_processor_count)
+    return "%s|sm%d|src=%s" % (p.name, p.multi_processor_count, build.library_digest())
 
 
 def _load() -> dict:

@@ -6,6 +6,7 @@ Run as ``python -m paper_1909_04750_gb300.build`` or call ``build()``.
 """
 from __future__ import annotations
 
+import functools
 import glob
 import hashlib
 import os
@@ -56,6 +57,13 @@ def sources_digest(names=("keystream_kernels.cu", "keystream_device.cuh",
                 if code:
                     h.update(code.encode() + b"\n")
     return h.hexdigest()[:16]
+
+
+@functools.lru_cache(maxsize=None)
+def library_digest() -> str:
+    """The digest of all kernel and host sources of the library."""
+    return sources_digest(tuple(sorted(os.path.basename(p) for p in _sources() + _headers()
+                                       if os.path.dirname(p) == CSRC)))
 
 
 def _newest(paths):
