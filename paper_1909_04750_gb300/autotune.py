@@ -4,7 +4,9 @@ For a (GPU, instance count, bits per call, layout) the library's
 ``mickey_tune`` times every compiled configuration -- grid, paired or
 two-block persistent launch, 2 or 4 clocks per inner step, and the output
 tile: direct 4-byte row stores or rows staged 2, 4 or 8 tiles deep (8-, 16-
-or 32-byte row chunks) -- on the handle's own streams (state saved and
+or 32-byte row chunks); for handles of up to 96 groups per SM also the launch
+the library takes by itself (a thread per instance, or four warps per 32
+groups) -- on the handle's own streams (state saved and
 restored) and keeps the fastest; among candidates within 1 % of it the
 deepest row staging wins (whole 32-byte sectors: the least DRAM traffic at
 the same speed).  The
@@ -88,8 +90,10 @@ def tune(streams, n_bits: int, layout: int, refresh: bool = False) -> dict:
 
 
 def describe(entry: dict) -> str:
+    if entry["mode"] == N.MODE_AUTO:     # has neither a step nor a staging depth to choose
+        return "auto, a thread per instance or four warps per 32 groups"
     st = entry["stage"]
-    default = {N.MODE_PERSISTENT: 8, N.MODE_AUTO: 8}.get(entry["mode"], 4)
+    default = {N.MODE_PERSISTENT: 8}.get(entry["mode"], 4)
     depth = default if st == 1 else st
     rows = "direct rows" if not st else ("staged rows" if depth == default
                                          else "rows staged %d tiles" % depth)

@@ -38,3 +38,11 @@ def test_the_digest_covers_every_source(tmp_path, monkeypatch):
     seen.add(build.library_digest())
     assert len(seen) == len(os.listdir(tmp_path / "csrc")) + 1
     build.library_digest.cache_clear()
+
+
+def test_the_librarys_own_launch_is_described_as_what_it_is():
+    from paper_1909_04750_gb300 import _native as N
+    own = autotune.describe({"mode": N.MODE_AUTO, "unroll": 4, "stage": 1})
+    assert "clocks/step" not in own and "staged" not in own and own.startswith("auto")
+    paired = autotune.describe({"mode": N.MODE_PERSISTENT, "unroll": 4, "stage": 1})
+    assert paired == "persistent, 4 clocks/step, staged rows"
