@@ -376,7 +376,8 @@ __device__ __forceinline__ void crc_byte(uint32_t (&c)[8], const uint32_t (&m)[8
   for (int j = 0; j < 8; ++j) c[j] = y[j];
 }
 
-// ANY: any length and alignment.  The warp reads the message's whole 16-byte
+// ANY: any alignment and any length from 31 bytes on (which has a whole aligned
+// unit; shorter messages take the table kernel).  The warp reads the message's whole 16-byte
 // aligned units, the last of them in lane 31 of the last chunk (units that a
 // message does not have count as zeros, which change nothing in front of it);
 // lane l takes message l's bytes before its first unit and behind its last
@@ -497,20 +498,15 @@ __global__ void __launch_bounds__(kCrcWarpBlock)
             (reinterpret_cast<uintptr_t>(first) + 15) & ~uintptr_t(15));
         const uint8_t *u1 =
             reinterpret_cast<const uint8_t *>(reinterpret_cast<uintptr_t>(end) & ~uintptr_t(15));
-        const bool units = u1 > u0;
-        uint32_t c = crc_bytes(table, init, first, units ? u0 : end);
-        if (units) {
-          const uint32_t k = past.k[size_t(u1 - u0) == (len & ~size_t(15)) ? 0 : 1];
-          uint32_t y = 0;                             // c k mod P
+        const uint32_t c = crc_bytes(table, init, first, u0);
+        const uint32_t k = past.k[size_t(u1 - u0) == (len & ~size_t(15)) ? 0 : 1];
+        uint32_t y = 0;                               // c k mod P
 #pragma unroll
-          for (int b = 7; b >= 0; --b) {
-            y = (y << 1) ^ ((y >> 7) & 1u ? 0x100u | poly : 0u);
-            y ^= (k >> b) & 1u ? c : 0u;
-          }
-          r = crc_bytes(table, r ^ y, u1, end);
-        } else {
-          r = c;
+        for (int b = 7; b >= 0; --b) {
+          y = (y << 1) ^ ((y >> 7) & 1u ? 0x100u | poly : 0u);
+          y ^= (k >> b) & 1u ? c : 0u;
         }
+        r = crc_bytes(table, r ^ y, u1, end);
       }
     }
     if (m0 + lane < n) crc[m0 + lane] = uint8_t(r ^ xorout);
@@ -628,7 +624,7 @@ uint32_t gf2_xpow(uint64_t e, uint32_t P) {
 CrcPast crc_past(uint8_t poly, size_t len) {
   const uint32_t P = 0x100u | poly;
   const uint64_t U = len / 16;
-  return CrcPast{{gf2_xpow(128 * U, P), U ? gf2_xpow(128 * (U - 1), P) : 1u}};
+  return CrcPast{{gf2_xpow(128 * U, P), gf2_xpow(128 * (U - 1), P)}};   // U > 0
 }
 
 CrcJoin crc_join_matrices(uint8_t poly) {
