@@ -25,9 +25,12 @@
  *           segment continuing a warp-group from the state its predecessor
  *           published (a bounded wait: MICKEY_SPIN_LIMIT polls of about 256
  *           ns, after which grain_sync reports MICKEY_E_TIMEOUT).  Handles
- *           with few groups (bitsliced up to 54 per SM, bytes up to 86 or any
- *           number when rows are not 16-byte aligned) run one thread per
- *           instance instead.  MICKEY_GRAIN_QUEUE, read when a handle is
+ *           with few groups run one thread per instance instead: bytes up to
+ *           86 per SM, or any number when rows of more than 4 bytes are not
+ *           16-byte aligned (rows of 1 or 4 bytes 32, of 2 or 3 bytes 64);
+ *           bitsliced up to 54, fewer for calls of few bits.  Other bitsliced
+ *           calls of up to 16 bits run a thread per group that only moves the
+ *           states.  MICKEY_GRAIN_QUEUE, read when a handle is
  *           created: 1 forces segments that wait for their predecessors
  *           whatever the number of groups, 0 the paired launch as above.
  */

@@ -212,14 +212,16 @@ MICKEY_API mickey_streams *mickey_import_state(const uint8_t *states,
  *           with an emission warp that transposes and stores its tiles; with
  *           at least as many 1024-instance warp-groups as clock warps the
  *           groups x tiles work line is cut into equal segments (one block
- *           per SM, cooperative), else each pair takes one whole warp-group;
+ *           per SM, cooperative where a warp-group is cut), else each pair
+ *           takes one whole warp-group;
  *           MICKEY_MODE_PERSISTENT2: two warps per SM sub-partition, each
  *           clocking and emitting (two blocks per SM, rows staged four
  *           tiles deep; with too few warp-groups it runs as PERSISTENT);
  *           MICKEY_MODE_AUTO: one thread per instance for handles of up to 18
  *           32-lane groups per SM (about 87,000 instances; up to 52 for rows of
- *           bytes that are not whole words), four warps per 32 groups for
- *           handles of up to 96 groups per SM (about 467,000 instances), else
+ *           bytes that are not whole words, up to 13 for calls of up to 8
+ *           bits), four warps per 32 groups for handles of up to 96 groups per
+ *           SM (about 467,000 instances), else
  *           as PERSISTENT; unroll and stage only matter there.
  *   unroll  clocks per inner step, 2 or 4.
  *   stage   the output tile of the row layouts: 0 writes each 32-clock tile's

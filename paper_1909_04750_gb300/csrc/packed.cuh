@@ -21,7 +21,7 @@
 // that can be a multiply-add goes to the FMA pipe: left shifts, the feedback
 // words k2 + fb (FB0 part) + fb cbs (FB1 part) (each bit a 0/1 times a
 // constant, differences mod 2^32), fb_R x RTAPS and cb_R x r_i.  That leaves
-// 22 logic and 23 multiply-add operations per clock of 32 instances.
+// 22 logic and 21 multiply-add operations per clock of 32 instances.
 // Measured (GB300, 2.07 GHz, with the row stores): 26.0 ns per clock for a lone
 // warp, 27.6 with one warp per SM sub-partition; clocks alone 782 Gbit/s with
 // eight (717 with the R update in logic operations).  The logic pipe would
