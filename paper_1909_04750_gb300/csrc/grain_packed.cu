@@ -13,7 +13,7 @@
 // each step and are back in place after five.
 //
 // Measured (GB300, us): 4001 instances x 20,002 bits with the initialisation
-// 1214 -> 82; 155,648 x 8192 bits of bytes 1025 -> 204 (6.3 Tbit/s); rows off
+// 1127 to 1488 -> 82; 155,648 x 8192 bits of bytes 1025 -> 204 (6.3 Tbit/s); rows off
 // the 16-byte grid, 2^20 x 1001 bits 1196 -> 216.  A lone warp takes 4.7 ns
 // per clock (9.7 cycles; its logic operations fill 4.9); at full occupancy
 // 6.8 Tbit/s, 0.82 of what the logic pipe allows for 38 operations per 16

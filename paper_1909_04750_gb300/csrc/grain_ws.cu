@@ -12,7 +12,7 @@
 // What bounds it: the logic pipe of a sub-partition, on which one clock warp
 // alone issues at 0.77 (94 cycles per clock for 72 of logic) when its body
 // fits the instruction cache, and the emission's 0.2 of that.  2^20 x 2^14
-// bits, a re-key and the call: bytes 2444 -> 1655 us, bitsliced 1750 -> 1320
+// bits, a re-key and the call: bytes 2444 -> 1621 us, bitsliced 1750 -> 1310
 // us against a warp per warp-group of 80-clock bodies with the emission in
 // its own instruction stream (those bodies did not fit, and the busiest
 // sub-partitions had two of 1024 chains where others had one; the segments

@@ -23,7 +23,7 @@
 // Bound by the logic pipe: the clocks of the longest lanes (0.76 of the clocked
 // bits are output below), then the emission warp's share of it.  Measured, 2^20
 // streams, lengths uniform in [2^13, 2^14], bytes at the packed offsets, call
-// by call: 21.9 -> 11.7 ms (1105 Gbit/s); before, one warp clocked, tested each
+// by call: 21.9 -> 11.3 ms (1145 Gbit/s); before, one warp clocked, tested each
 // clock for ends and emitted with byte stores.
 #include "keystream_persistent.cuh"
 #include "packed.cuh"
