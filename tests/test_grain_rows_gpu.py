@@ -61,5 +61,5 @@ def test_partial_last_tile_costs_no_more_stores():
             st.generate(n_bits, "bytes", out=out)
         e1.record()
         e1.synchronize()
-        ms[n_bits] = e0.elapsed_time(e1)            # the second round's
+        ms[n_bits] = e0.elapsed_time(e1)            # of the second turn
     assert ms[4092] < 2 * ms[4096], ms
