@@ -209,11 +209,12 @@ void grain_release(grain_streams *s) {
 //   groups                       126      7296      9728      14592      32768
 //   bitsliced, 8192 bits      40, 388   343, 390  454, 390  672, 389   -, 661
 //   bytes, 8192 bits          41, 506   290, 514  380, 509  561, 517  1265, 818
-//   initialisation            11, 28    18, 27    21, 27     25, 30     44, 35
+//   initialisation            11, 28    18, 27    21, 27     25, 27     44, 35
+//   (the initialisation is level at 15,625: 26, 26; at 19,456: 30, 27)
 // The packed launches' work grows with the groups from one warp per SM
 // sub-partition on; a thread per group takes one warp-group's chain until
 // every sub-partition has one (19456 groups; the initialisation: two).
-constexpr uint32_t kGrainPackedInitPerSm = 128;
+constexpr uint32_t kGrainPackedInitPerSm = 102;
 constexpr uint32_t kGrainPackedBitslicedPerSm = 54, kGrainPackedBytesPerSm = 86;
 // Short calls are moving states, which costs a thread per instance its
 // transposes, 1.6 us per 1000 groups (us; packed, thread per group):

@@ -35,10 +35,10 @@ def _sample(n, k=600):
 
 
 # Grain: groups per SM at the lines of short rows (32, 64), of bitsliced calls
-# whose line moves with the clocks (30, 50), and above all of them; every kind of
-# row on and off the grid, at an aligned output and an odd one
+# whose line moves with the clocks (30, 50), of the loading (102), and above all;
+# every kind of row on and off the grid, at an aligned output and an odd one
 @pytest.mark.parametrize("per_sm,extra", [(30, 0), (32, 0), (32, 1), (50, 0), (64, 0), (64, 1),
-                                          (140, 3)])
+                                          (102, 0), (102, 1), (140, 3)])
 def test_grain_short_calls(per_sm, extra):
     from oracle import grain as og
     from paper_1909_04750_gb300.grain import GrainStreams
